@@ -67,7 +67,10 @@ typedef enum { LB_BC_PERIODIC = 0, LB_BC_COUETTE = 1 } lb_bc;
  * Observables are reduced in FP64. */
 typedef enum { LB_FP32 = 0, LB_FP16_SHIFTED = 1, LB_FP64 = 2, LB_FP16_SHIFTED_SR = 3 } lb_precision;
 
-/* Kernel family: AUTO picks TILED when the shape allows it, else GENERIC. */
+/* Kernel family: AUTO picks TILED when the shape allows it, else GENERIC.  Under
+ * AUTO lb_step advances a small lattice (2^17 sites over all cells) with a kernel
+ * that takes many steps per launch; the family AUTO picked then serves steps
+ * inside a capture of the caller's and is what lb_get_kernel reports. */
 typedef enum { LB_KERNEL_AUTO = 0, LB_KERNEL_GENERIC = 1, LB_KERNEL_TILED = 2 } lb_kernel;
 
 /* One lattice cell, in the paper's symbols.  All cells of a handle share nx, ny
@@ -210,8 +213,8 @@ lb_status lb_reductions(lb_handle* h, double* mass_ab, double* momentum_xy);
  * ignores both.  LB_ERR_UNSUPPORTED if the shape does not allow the request. */
 lb_status lb_set_kernel(lb_handle* h, lb_kernel kernel, int tile_x, int tile_y);
 
-/* Times the supported tiles on this handle's buffers (the state is left
- * unchanged) and selects the fastest.  cache_path (nullable): a text file where
+/* Times the supported tiles (and what AUTO runs on a small lattice) on this
+ * handle's buffers (the state is left unchanged) and selects the fastest.  cache_path (nullable): a text file where
  * results are looked up and stored, keyed by device, shape, cell count and
  * precision.  Synchronous. */
 lb_status lb_autotune(lb_handle* h, const char* cache_path);

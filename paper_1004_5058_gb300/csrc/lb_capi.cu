@@ -67,6 +67,7 @@ struct lb_handle {
     lb_kernel kernel = LB_KERNEL_GENERIC;
     int tile_x = 0, tile_y = 0;
     TiledPlan* plan = nullptr;
+    PatchPlan* patch = nullptr;  // small lattices under LB_KERNEL_AUTO: lb_step runs this one
     long long launches = 0;
     int inject = 0;  // lb_test_inject: 1 = stalled row copy, 2 = failed launch (next lb_step)
     std::string last_error;
@@ -112,6 +113,7 @@ static void release(lb_handle* h)
     if (h->stream) cudaStreamSynchronize(h->stream);
     free_graphs(h);
     if (h->plan) tiled_destroy(h->plan);
+    patch_destroy(h->patch);
     cudaFree(h->f[0]);
     cudaFree(h->f[1]);
     cudaFree(h->aux);
@@ -242,18 +244,51 @@ static lb_status reset_counters(lb_handle* h)
     return LB_OK;
 }
 
+static lb_status select_kernel(lb_handle* h, lb_kernel k, int tx, int ty);
+
+// The kernel family and tile of LB_KERNEL_AUTO.
+static lb_status select_by_shape(lb_handle* h)
+{
+    // the widest tile that divides nx, else the widest that fits (a narrower
+    // last strip), else the generic kernel
+    const int txs[] = {128, 64, 32};
+    for (int pass = 0; pass < 2; ++pass)
+        for (int c : txs)
+            if ((pass == 1 || h->nx % c == 0) && tiled_supported(h->gbuf, h->elem, c, 0) &&
+                select_kernel(h, LB_KERNEL_TILED, c, 0) == LB_OK)
+                return LB_OK;
+    return select_kernel(h, LB_KERNEL_GENERIC, 0, 0);
+}
+
+static void drop_patch(lb_handle* h)
+{
+    patch_destroy(h->patch);
+    h->patch = nullptr;
+}
+
+// Under LB_KERNEL_AUTO a small lattice steps through the patch kernel.  us per
+// step, the kernel of select_by_shape against the patch kernel (one cell):
+//   FP32  64^2 9.3 / 3.2, 128^2 10.4 / 3.4, 256^2 10.4 / 6.0, 384^2 10.5 / 9.7, 512^2 12.3 / 16.1;
+//   FP64  64^2 102 / 12.3, 128^2 114 / 18.5, 256^2 114 / 62, 384^2 115 / 120;
+//   37 x 23 (generic pair) FP32 5.5 / 3.6, 301 x 243 FP32 10.1 / 9.0;
+//   101 x 83 (generic pair) FP64 27 / 12.9, 201 x 163 FP64 26.9 / 33.9.
+// The tiled kernel's time hardly depends on the size up to 2^17 sites (its rows
+// are a serial chain), the patch kernel's grows with it; they meet near there, and
+// with the FP64 generic pair, which spreads over the chip as well, near 2^15.
+static void select_patch(lb_handle* h)
+{
+    const long long most = h->kernel == LB_KERNEL_GENERIC && h->prec == LB_FP64 ? 1LL << 15 : 1LL << 17;
+    if (h->slab || (long long)h->n_cells * h->nx * h->ny > most) return;
+    h->patch = patch_create(h->g, (int)h->prec, h->bc);
+    if (h->patch) patch_set_collision(h->patch, collision_kind(h->cells));
+}
+
 static lb_status select_kernel(lb_handle* h, lb_kernel k, int tx, int ty)
 {
     if (k == LB_KERNEL_AUTO) {
-        // the widest tile that divides nx, else the widest that fits (a narrower
-        // last strip), else the generic kernel
-        const int txs[] = {128, 64, 32};
-        for (int pass = 0; pass < 2; ++pass)
-            for (int c : txs)
-                if ((pass == 1 || h->nx % c == 0) && tiled_supported(h->gbuf, h->elem, c, 0) &&
-                    select_kernel(h, LB_KERNEL_TILED, c, 0) == LB_OK)
-                    return LB_OK;
-        return select_kernel(h, LB_KERNEL_GENERIC, 0, 0);
+        const lb_status st = select_by_shape(h);
+        if (st == LB_OK) select_patch(h);
+        return st;
     }
     if (k == LB_KERNEL_GENERIC && h->slab)
         return fail(h, LB_ERR_UNSUPPORTED, "lb_set_kernel: a slab runs the tiled kernel only");
@@ -263,6 +298,7 @@ static lb_status select_kernel(lb_handle* h, lb_kernel k, int tx, int ty)
             tiled_destroy(h->plan);
             h->plan = nullptr;
         }
+        drop_patch(h);
         h->kernel = LB_KERNEL_GENERIC;
         h->tile_x = 32;
         h->tile_y = 8;
@@ -287,6 +323,7 @@ static lb_status select_kernel(lb_handle* h, lb_kernel k, int tx, int ty)
     if (!p) return fail(h, LB_ERR_UNSUPPORTED, "lb_set_kernel: %s", msg ? msg : "tiled plan failed");
     tiled_set_collision(p, collision_kind(h->cells));
     if (h->plan) tiled_destroy(h->plan);
+    drop_patch(h);
     h->plan = p;
     h->kernel = LB_KERNEL_TILED;
     tiled_tiles(p, &h->tile_x, &h->tile_y);
@@ -784,6 +821,46 @@ static cudaError_t run_chunk(lb_handle* h, int src, int steps, bool sample_last,
     return cudaGraphLaunch(it->second, h->stream);
 }
 
+// true while the stream is being captured into a graph of the caller's (where a
+// cooperative launch is left out)
+static bool capturing(cudaStream_t st)
+{
+    cudaStreamCaptureStatus c = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(st, &c) != cudaSuccess) {
+        cudaGetLastError();
+        return true;
+    }
+    return c != cudaStreamCaptureStatusNone;
+}
+
+// Steps of a small lattice: launches of up to 512 steps (one or two milliseconds,
+// so that other streams' kernels get their turn).
+static cudaError_t patch_steps(lb_handle* h, long long n_steps, int* nl)
+{
+    for (long long done = 0; done < n_steps;) {
+        const int piece = (int)std::min<long long>(n_steps - done, 512);
+        int first = -1;  // first sampled step of this piece
+        long long samples = 0;
+        if (h->every > 0) {
+            const long long t = h->t, k = t <= h->start ? 0 : (t - h->start + h->every - 1) / h->every;
+            const long long next = h->start + k * h->every - t;
+            if (next < piece) {
+                first = (int)next;
+                samples = (piece - 1 - next) / h->every + 1;
+            }
+        }
+        const cudaError_t e = launch_patch_steps(h->patch, h->f[h->cur], h->f[h->cur ^ 1], piece, first,
+                                                 (int)std::min<long long>(h->every, 1 << 30), true, h->d_cells,
+                                                 h->acc_prof, h->acc_wall, h->d_err, h->stream, nl);
+        if (e != cudaSuccess) return e;
+        h->cur ^= piece & 1;
+        h->t += piece;
+        h->n_samples += samples;
+        done += piece;
+    }
+    return cudaSuccess;
+}
+
 lb_status lb_step(lb_handle* h, long long n_steps)
 {
     Trace trace("lb_step");
@@ -810,6 +887,14 @@ lb_status lb_step(lb_handle* h, long long n_steps)
     }
     int nl = 0;
     long long done = 0;
+    if (h->patch && h->inject != 1 && !capturing(h->stream)) {
+        const cudaError_t e = patch_steps(h, n_steps, &nl);
+        if (e != cudaSuccess) {
+            cudaGetLastError();
+            return fail(h, LB_ERR_CUDA, "lb_step: launch failed: %s", cudaGetErrorString(e));
+        }
+        done = n_steps;
+    }
     while (done < n_steps) {
         // steps up to and including the next sampled step (or the end)
         long long left = n_steps - done;
@@ -1039,6 +1124,7 @@ lb_status lb_autotune(lb_handle* h, const char* cache_path)
     }
     // candidates: generic, and every supported tile
     std::vector<std::tuple<int, int, int>> cand;
+    cand.emplace_back((int)LB_KERNEL_AUTO, 0, 0);  // the patch kernel, where it serves the lattice
     cand.emplace_back((int)LB_KERNEL_GENERIC, 0, 0);
     const int txs[] = {32, 64, 128, 256};
     const int tys[] = {0, 16, 32, 64};  // 0: segment height from the fill model
@@ -1049,17 +1135,26 @@ lb_status lb_autotune(lb_handle* h, const char* cache_path)
     CK(h, cudaEventCreate(&e0));
     CK(h, cudaEventCreate(&e1));
     float best = 1e30f;
-    std::tuple<int, int, int> best_c = cand[0];
-    const int reps = 6;
+    std::tuple<int, int, int> best_c = cand[1];
+    const int reps = 6, patch_reps = 64;  // the patch kernel takes many steps per launch
     for (auto& c : cand) {
         if (select_kernel(h, (lb_kernel)std::get<0>(c), std::get<1>(c), std::get<2>(c)) != LB_OK) continue;
+        const bool patch = std::get<0>(c) == LB_KERNEL_AUTO;
+        if (patch && !h->patch) continue;
         int nl = 0;
         // trial steps read the current buffer and write the other one, without
         // swapping, so the state is unchanged
-        bool ok = true;
-        for (int r = 0; r < 2 && ok; ++r) ok = enqueue_one_step(h, h->cur, false, &nl) == cudaSuccess;
+        auto trial = [&](int n) {
+            if (patch)
+                return launch_patch_steps(h->patch, h->f[h->cur], h->f[h->cur ^ 1], n * patch_reps / reps, -1, 0, false,
+                                          h->d_cells, h->acc_prof, h->acc_wall, h->d_err, h->stream, &nl) == cudaSuccess;
+            for (int r = 0; r < n; ++r)
+                if (enqueue_one_step(h, h->cur, false, &nl) != cudaSuccess) return false;
+            return true;
+        };
+        bool ok = trial(2);
         cudaEventRecord(e0, h->stream);
-        for (int r = 0; r < reps && ok; ++r) ok = enqueue_one_step(h, h->cur, false, &nl) == cudaSuccess;
+        ok = ok && trial(reps);
         cudaEventRecord(e1, h->stream);
         if (!ok || cudaEventSynchronize(e1) != cudaSuccess) {
             cudaGetLastError();
@@ -1068,6 +1163,7 @@ lb_status lb_autotune(lb_handle* h, const char* cache_path)
         h->launches += nl;
         float ms = 0.f;
         cudaEventElapsedTime(&ms, e0, e1);
+        if (patch) ms *= (float)reps / patch_reps;
         if (ms < best) {
             best = ms;
             best_c = c;
@@ -1258,6 +1354,7 @@ lb_status lb_load(lb_handle* h, const char* path)
     h->h_err[0] = 0;
     h->cells = cells;
     if (h->plan) tiled_set_collision(h->plan, collision_kind(h->cells));
+    if (h->patch) patch_set_collision(h->patch, collision_kind(h->cells));
     free_graphs(h);  // captured launches may name the other kernel family
     h->cur = 0;
     h->t = hd.t;

@@ -40,6 +40,21 @@ void tiled_inject_skip(TiledPlan* p, uint32_t row);
 enum { TILED_BGK_ONE_TIME = 0, TILED_BGK = 1, TILED_MRT = 2 };
 void tiled_set_collision(TiledPlan* p, int collision);
 
+// patch kernel (lb_patch.cu): many steps of a small lattice in one cooperative
+// launch, for whole cells of any width
+struct PatchPlan;
+// nullptr where the device, the shape or memory does not allow it.
+PatchPlan* patch_create(const Geom& g, int prec, int bc);
+void patch_destroy(PatchPlan* p);
+void patch_set_collision(PatchPlan* p, int collision);
+// `steps` steps from src, ping-ponging with dst (swap), or reading src and writing
+// dst every time (timing a kernel without changing the state).  Sampled steps:
+// first, first + every, ... counted from this launch's first step (first < 0:
+// none); their sums are added to acc_prof and acc_wall.
+cudaError_t launch_patch_steps(PatchPlan* p, void* src, void* dst, int steps, int first, int every, bool swap,
+                               const CellDev* cells, double* acc_prof, double* acc_wall, unsigned* err,
+                               cudaStream_t st, int* n_launches);
+
 // auxiliary kernels (lb_aux.cu)
 template <class T>
 cudaError_t launch_equilibrium(const double* src, T* f, const Geom& g, const CellDev* cells, cudaStream_t st);

@@ -30,6 +30,7 @@
 #include <type_traits>
 
 #include "lb_internal.h"
+#include "lb_pair.cuh"
 #include "lbhb.h"
 #include "tma.cuh"
 
@@ -82,119 +83,6 @@ __host__ __device__ constexpr int ring_depth(int tx, int elem)
 __host__ __device__ constexpr int ring_species_stride(int tx)
 {
     return RING * (tx + 4) + ((16 - (RING * (tx + 4)) % 32) + 32) % 32;
-}
-
-// Two adjacent columns of one species per thread: vector (8-byte for FP32)
-// shared-memory accesses and two independent sites per thread.
-template <class T> struct Vec2;
-template <> struct Vec2<float> {
-    __device__ static void ld(const float* p, float& a, float& b)
-    {
-        const float2 v = *reinterpret_cast<const float2*>(p);
-        a = v.x;
-        b = v.y;
-    }
-    __device__ static void st(float* p, float a, float b) { *reinterpret_cast<float2*>(p) = make_float2(a, b); }
-};
-template <> struct Vec2<double> {
-    __device__ static void ld(const double* p, double& a, double& b)
-    {
-        const double2 v = *reinterpret_cast<const double2*>(p);
-        a = v.x;
-        b = v.y;
-    }
-    __device__ static void st(double* p, double a, double b) { *reinterpret_cast<double2*>(p) = make_double2(a, b); }
-};
-template <> struct Vec2<__half> {
-    __device__ static void ld(const __half* p, float& a, float& b)
-    {
-        const __half2 v = *reinterpret_cast<const __half2*>(p);
-        a = __low2float(v);
-        b = __high2float(v);
-    }
-    // FP16 storage of shifted values: the caller subtracts the shift
-    __device__ static void st(__half* p, float a, float b) { *reinterpret_cast<__half2*>(p) = __floats2half2_rn(a, b); }
-};
-// stochastically rounded FP16: loads as for __half (the caller unscales),
-// stores with the thread's dither stream
-template <> struct Vec2<half_sr> {
-    __device__ static void ld(const half_sr* p, float& a, float& b)
-    {
-        const __half2 v = *reinterpret_cast<const __half2*>(p);
-        a = __low2float(v);
-        b = __high2float(v);
-    }
-    __device__ static void st(half_sr* p, float a, float b, Dither& d)
-    {
-        const __half lo = half_sr_round(a, d), hi = half_sr_round(b, d);
-        *reinterpret_cast<__half2*>(p) = __halves2half2(lo, hi);
-    }
-};
-// paired and single stores of values already in the stored representation,
-// dithered where the storage asks for it
-template <class T, class C>
-__device__ inline void st_pair(T* p, C a, C b, Dither& d)
-{
-    if constexpr (Store<T>::dithered)
-        Vec2<T>::st(p, a, b, d);
-    else
-        Vec2<T>::st(p, a, b);
-}
-template <class T, class C>
-__device__ inline void st_one(T* p, C v, Dither& d)
-{
-    if constexpr (std::is_same<T, half_sr>::value)
-        p->h = half_sr_round(v, d);
-    else if constexpr (std::is_same<T, __half>::value)
-        *p = __float2half_rn(v);
-    else
-        *p = v;
-}
-
-// Element CI (0..5) of a window row of six columns held as three lane pairs.
-template <int CI, class C>
-__device__ __forceinline__ C win_at(const P2<C> (&row)[3])
-{
-    return (CI & 1) ? row[CI >> 1].b() : row[CI >> 1].a();
-}
-
-// g(r + c) - g(r - c) of Eq. (FFF) for both sites of a thread, c = (DX, DY):
-// site o sits at column 2 + o of window row MID.  Pairs at an even column
-// offset are the stored pairs (one packed subtraction); odd offsets straddle
-// two pairs (two scalar subtractions).
-template <int DX, int DY, int MID, int NR, class C>
-__device__ __forceinline__ P2<C> pair_diff(const P2<C> (&w)[NR][3])
-{
-    constexpr int cp = 2 + DX, cm = 2 - DX;
-    if constexpr ((DX & 1) == 0)
-        return w[MID + DY][cp / 2] - w[MID - DY][cm / 2];
-    else
-        return P2<C>(win_at<cp>(w[MID + DY]) - win_at<cm>(w[MID - DY]),
-                     win_at<cp + 1>(w[MID + DY]) - win_at<cm + 1>(w[MID - DY]));
-}
-
-// The half-stencil differences of psi (window rows k-2..k+2) and of the partner
-// density rho_s' (rows k-1..k+1, belt 1 only), in the order of hs_dx / hs_dy.
-template <class C>
-__device__ __forceinline__ void window_diffs(const P2<C> (&v)[5][3], const P2<C> (&e)[3][3], P2<C> d[12],
-                                             P2<C> de[4])
-{
-    d[0] = pair_diff<hs_dx(0), hs_dy(0), 2>(v);
-    d[1] = pair_diff<hs_dx(1), hs_dy(1), 2>(v);
-    d[2] = pair_diff<hs_dx(2), hs_dy(2), 2>(v);
-    d[3] = pair_diff<hs_dx(3), hs_dy(3), 2>(v);
-    d[4] = pair_diff<hs_dx(4), hs_dy(4), 2>(v);
-    d[5] = pair_diff<hs_dx(5), hs_dy(5), 2>(v);
-    d[6] = pair_diff<hs_dx(6), hs_dy(6), 2>(v);
-    d[7] = pair_diff<hs_dx(7), hs_dy(7), 2>(v);
-    d[8] = pair_diff<hs_dx(8), hs_dy(8), 2>(v);
-    d[9] = pair_diff<hs_dx(9), hs_dy(9), 2>(v);
-    d[10] = pair_diff<hs_dx(10), hs_dy(10), 2>(v);
-    d[11] = pair_diff<hs_dx(11), hs_dy(11), 2>(v);
-    de[0] = pair_diff<hs_dx(0), hs_dy(0), 1>(e);
-    de[1] = pair_diff<hs_dx(1), hs_dy(1), 1>(e);
-    de[2] = pair_diff<hs_dx(2), hs_dy(2), 1>(e);
-    de[3] = pair_diff<hs_dx(3), hs_dy(3), 1>(e);
 }
 
 // Threads per CTA: a thread per (species, column pair), TX threads, plus one
