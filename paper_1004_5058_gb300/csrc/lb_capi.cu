@@ -159,6 +159,17 @@ static void fill(ParamSet<C>& d, const lb_cell_params& c)
     d.g1[1] = C(c.g_bb1);
     d.g2[0] = C(c.g_aa2);
     d.g2[1] = C(c.g_bb2);
+    // couplings folded into the stencil weights (Couplings<V, double>)
+    const double g1[2] = {c.g_aa1, c.g_bb1}, g2[2] = {c.g_aa2, c.g_bb2};
+    for (int s = 0; s < 2; ++s) {
+        d.gc[s][0] = C(g1[s] * hs_w1(0) + g2[s] * hs_w2(0));
+        d.gc[s][1] = C(g1[s] * hs_w1(2) + g2[s] * hs_w2(2));
+        d.gc[s][2] = C(g2[s] * 2.0 * hs_w2(4));
+        d.gc[s][3] = C(g2[s] * hs_w2(6));
+        d.gc[s][4] = C(g2[s] * 2.0 * hs_w2(10));
+    }
+    d.xc[0] = C(c.g_ab / c.rho0 * hs_w1(0));
+    d.xc[1] = C(c.g_ab / c.rho0 * hs_w1(2));
     d.u_wall = C(c.u_wall);
     d.f0 = C(c.f0);
     d.two_over_ny = C(2.0 / c.ny);
@@ -269,16 +280,16 @@ static void drop_patch(lb_handle* h)
 // Under LB_KERNEL_AUTO a small lattice steps through the patch kernel.  us per
 // step, the kernel of select_by_shape against the patch kernel (one cell):
 //   FP32  64^2 9.3 / 3.2, 128^2 10.4 / 3.4, 256^2 10.4 / 6.0, 384^2 10.5 / 9.7, 512^2 12.3 / 16.1;
-//   FP64  64^2 102 / 12.3, 128^2 114 / 18.5, 256^2 114 / 62, 384^2 115 / 120;
+//   FP64  64^2 84 / 11, 128^2 97 / 14, 256^2 97 / 45, 320^2 100 / 75, 360^2 102 / 100;
 //   37 x 23 (generic pair) FP32 5.5 / 3.6, 301 x 243 FP32 10.1 / 9.0;
-//   101 x 83 (generic pair) FP64 27 / 12.9, 201 x 163 FP64 26.9 / 33.9.
+//   101 x 83 (generic pair) FP64 24 / 12, 201 x 163 FP64 24.4 / 26.5.
 // The tiled kernel's time hardly depends on the size up to 2^17 sites (its rows
 // are a serial chain), the patch kernel's grows with it; they meet near there, and
 // with the FP64 generic pair, which spreads over the chip as well, near 2^15.
 static void select_patch(lb_handle* h)
 {
     const long long most = h->kernel == LB_KERNEL_GENERIC && h->prec == LB_FP64 ? 1LL << 15 : 1LL << 17;
-    if (h->slab || (long long)h->n_cells * h->nx * h->ny > most) return;
+    if (h->slab || (long long)h->n_cells * h->nx * h->ny >= most) return;
     h->patch = patch_create(h->g, (int)h->prec, h->bc);
     if (h->patch) patch_set_collision(h->patch, collision_kind(h->cells));
 }
@@ -838,20 +849,22 @@ static bool capturing(cudaStream_t st)
 static cudaError_t patch_steps(lb_handle* h, long long n_steps, int* nl)
 {
     for (long long done = 0; done < n_steps;) {
-        const int piece = (int)std::min<long long>(n_steps - done, 512);
-        int first = -1;  // first sampled step of this piece
+        int piece = (int)std::min<long long>(n_steps - done, 512);
+        int first = -1, every = 0;  // first sampled step of this piece
         long long samples = 0;
         if (h->every > 0) {
             const long long t = h->t, k = t <= h->start ? 0 : (t - h->start + h->every - 1) / h->every;
             const long long next = h->start + k * h->every - t;
             if (next < piece) {
                 first = (int)next;
-                samples = (piece - 1 - next) / h->every + 1;
+                every = (int)std::min<long long>(h->every, 1 << 30);
+                samples = std::min<long long>((piece - 1 - next) / every + 1, patch_max_samples(h->patch));
+                piece = (int)std::min<long long>(piece, next + samples * every);
             }
         }
-        const cudaError_t e = launch_patch_steps(h->patch, h->f[h->cur], h->f[h->cur ^ 1], piece, first,
-                                                 (int)std::min<long long>(h->every, 1 << 30), true, h->d_cells,
-                                                 h->acc_prof, h->acc_wall, h->d_err, h->stream, nl);
+        const cudaError_t e = launch_patch_steps(h->patch, h->f[h->cur], h->f[h->cur ^ 1], piece, first, every, true,
+                                                 h->tile_x, h->d_cells, h->acc_prof, h->acc_wall, h->d_err, h->stream,
+                                                 nl);
         if (e != cudaSuccess) return e;
         h->cur ^= piece & 1;
         h->t += piece;
@@ -1147,7 +1160,7 @@ lb_status lb_autotune(lb_handle* h, const char* cache_path)
         auto trial = [&](int n) {
             if (patch)
                 return launch_patch_steps(h->patch, h->f[h->cur], h->f[h->cur ^ 1], n * patch_reps / reps, -1, 0, false,
-                                          h->d_cells, h->acc_prof, h->acc_wall, h->d_err, h->stream, &nl) == cudaSuccess;
+                                          h->tile_x, h->d_cells, h->acc_prof, h->acc_wall, h->d_err, h->stream, &nl) == cudaSuccess;
             for (int r = 0; r < n; ++r)
                 if (enqueue_one_step(h, h->cur, false, &nl) != cudaSuccess) return false;
             return true;

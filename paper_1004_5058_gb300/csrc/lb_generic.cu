@@ -67,7 +67,7 @@ __global__ void __launch_bounds__(256) fused_generic_kernel(const T* __restrict_
         const long long k0 = (long long)y * g.nx + x;
         C rho[2] = {rho_f[k0], rho_f[n + k0]};
         C psi[2] = {rho_f[2 * n + k0], rho_f[3 * n + k0]};
-        Sums<C> sm[2];
+        Pull<C> pu[2];
 #pragma unroll
         for (int s = 0; s < 2; ++s) {
             C dpsi[12], drho[4];
@@ -79,10 +79,10 @@ __global__ void __launch_bounds__(256) fused_generic_kernel(const T* __restrict_
                 dpsi[k] = rho_f[(2 + s) * n + kp] - rho_f[(2 + s) * n + km];
                 if (k < 4) drho[k] = rho_f[(1 - s) * n + kp] - rho_f[(1 - s) * n + km];
             }
-            sm[s] = stencil_sums<C>(dpsi, drho);
+            pu[s] = Couplings<C>(p, s).pull(dpsi, drho);
         }
         Collided<C> c;
-        collide_site<C>(f, rho, psi, sm, p, body_force_x<C>(p, y), c);
+        collide_site<C>(f, rho, psi, pu, p, body_force_x<C>(p, y), c);
 
         const C u_top = p.u_wall, u_bot = -p.u_wall;
         Dither dz;  // stochastic rounding stream of this site (dithered storage only)

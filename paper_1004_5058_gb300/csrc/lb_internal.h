@@ -50,8 +50,10 @@ void patch_set_collision(PatchPlan* p, int collision);
 // `steps` steps from src, ping-ponging with dst (swap), or reading src and writing
 // dst every time (timing a kernel without changing the state).  Sampled steps:
 // first, first + every, ... counted from this launch's first step (first < 0:
-// none); their sums are added to acc_prof and acc_wall.
-cudaError_t launch_patch_steps(PatchPlan* p, void* src, void* dst, int steps, int first, int every, bool swap,
+// none, and at most patch_max_samples); their sums are added to acc_prof and
+// acc_wall in the order of a tiled kernel of tile_x columns.
+int patch_max_samples(const PatchPlan* p);
+cudaError_t launch_patch_steps(PatchPlan* p, void* src, void* dst, int steps, int first, int every, bool swap, int tile_x,
                                const CellDev* cells, double* acc_prof, double* acc_wall, unsigned* err,
                                cudaStream_t st, int* n_launches);
 

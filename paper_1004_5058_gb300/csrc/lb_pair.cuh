@@ -122,4 +122,43 @@ __device__ __forceinline__ void window_diffs(const P2<C> (&v)[5][3], const P2<C>
     de[3] = pair_diff<hs_dx(3), hs_dy(3), 1>(e);
 }
 
+// Sum of the u_x of a 32-column group of one row by 32 / NW adjacent lanes of a
+// warp, NW consecutive columns each (at(q): a lane's columns), in the first of
+// them; one fixed order for every kernel that samples.  FP32 values are carried
+// as an unevaluated (hi, lo) pair (error-free two-sum), ~2^-48 relative.
+template <int NW, class At> __device__ __forceinline__ double group_sum(int lane, At at)
+{
+    constexpr int SEG = 32 / NW;
+    using C = decltype(at(0));
+    if constexpr (sizeof(C) == 4) {
+        float hi = at(0), lo = 0.f;
+#pragma unroll
+        for (int q = 1; q < NW; ++q) {
+            const float v = at(q);
+            const float sum = __fadd_rn(hi, v);
+            const float bp = __fsub_rn(sum, hi);
+            lo = __fadd_rn(lo, __fadd_rn(__fsub_rn(hi, __fsub_rn(sum, bp)), __fsub_rn(v, bp)));
+            hi = sum;
+        }
+#pragma unroll
+        for (int o = SEG / 2; o > 0; o >>= 1) {
+            const float h2 = __shfl_down_sync(0xffffffffu, hi, o, SEG);
+            const float l2 = __shfl_down_sync(0xffffffffu, lo, o, SEG);
+            const float sum = __fadd_rn(hi, h2);
+            const float bp = __fsub_rn(sum, hi);
+            const float err = __fadd_rn(__fsub_rn(hi, __fsub_rn(sum, bp)), __fsub_rn(h2, bp));
+            hi = sum;
+            lo = __fadd_rn(__fadd_rn(lo, l2), err);
+        }
+        return (double)hi + (double)lo;
+    } else {
+        double v = 0.0;
+#pragma unroll
+        for (int q = 0; q < NW; ++q) v += at(q);
+#pragma unroll
+        for (int o = SEG / 2; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o, SEG);
+        return v;
+    }
+}
+
 }  // namespace lbhb

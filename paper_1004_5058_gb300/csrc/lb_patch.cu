@@ -24,7 +24,7 @@
 // -> stores -> flag, two trips through L2 and a release that waits for the stores:
 // 3.2 us at 64^2 FP32 (9.3 us as a launch of the tiled kernel per step).  FP64 is
 // bound by the FP64 pipe (64 cycles per warp instruction on each sub-partition):
-// 12.3 us at 64^2, 102 us before; two sites per thread took 19.3 us.
+// 11 us at 64^2, 102 us before; two sites per thread took 19.3 us where one took 12.3.
 //
 // Steps are ordered by one flag per patch (the number of steps it has behind it):
 // a patch starts step s when all patches within three sites of it have finished
@@ -50,8 +50,10 @@ struct PatchArgs {
     int steps;
     int first, every;  // sampled steps of this launch: first, first + every, ... (first < 0: none)
     const CellDev* cells;
-    double* prof;   // [cell][npx][ny] sums of u_x over the patch's columns, over the sampled steps
-    double* wall;   // [cell][npx][2]  sums of Pi_top, Pi_bot
+    // sampled steps k = 0, 1, ... of this launch, in the compute type: u_x of every
+    // site [k][cell][ny][nx], and what the walls deliver [k][cell][top, bottom]
+    // [species][PatchLane::DW][columns / sites per lane]
+    void *u, *dp;
     unsigned* err;
     unsigned* flags;  // [cell][npy][npx] steps done
 };
@@ -83,21 +85,22 @@ __device__ __forceinline__ float ld_one(const half_sr* p) { return half_one(__ld
 template <class T> struct PatchLane {
     using V = P2<float>;
     static constexpr int NS = 2;
+    static constexpr int DW = 1;  // wall momentum of the pair, three links summed
 };
 template <> struct PatchLane<double> {
-    using V = double;
+    using V = P1;
     static constexpr int NS = 1;
+    static constexpr int DW = 3;  // of each link, so that pairs of sites can be summed link by link
 };
-__device__ __forceinline__ double first(double v) { return v; }
+__device__ __forceinline__ double first(P1 v) { return v.x; }
 __device__ __forceinline__ float first(P2<float> v) { return v.a(); }
-__device__ __forceinline__ double second(double v) { return v; }
+__device__ __forceinline__ double second(P1 v) { return v.x; }
 __device__ __forceinline__ float second(P2<float> v) { return v.b(); }
-__device__ __forceinline__ double from_partner(double v) { return __shfl_xor_sync(0xffffffffu, v, 16); }
+__device__ __forceinline__ P1 from_partner(P1 v) { return P1(__shfl_xor_sync(0xffffffffu, v.x, 16)); }
 __device__ __forceinline__ P2<float> from_partner(P2<float> v)
 {
     return P2<float>(__shfl_xor_sync(0xffffffffu, v.a(), 16), __shfl_xor_sync(0xffffffffu, v.b(), 16));
 }
-__device__ __forceinline__ double lane_psi(double rho, double rho0, double inv_rho0) { return psi_of(rho, rho0, inv_rho0); }
 
 // The half-stencil differences of psi and of the partner's density around one
 // lane, read from shared memory: ps and ro point at the window's first element
@@ -118,16 +121,16 @@ template <int W> __device__ __forceinline__ void lane_window(const float* ps, co
     *rho_p = e[1][1];
     window_diffs(v, e, d, de);
 }
-template <int W> __device__ __forceinline__ void lane_window(const double* ps, const double* ro, double d[12],
-                                                            double de[4], double* psi, double* rho_p)
+template <int W> __device__ __forceinline__ void lane_window(const double* ps, const double* ro, P1 d[12], P1 de[4],
+                                                            P1* psi, P1* rho_p)
 {
-    *psi = ps[2 * W + 2];
-    *rho_p = ro[W + 2];
+    *psi = P1(ps[2 * W + 2]);
+    *rho_p = P1(ro[W + 2]);
 #pragma unroll
     for (int k = 0; k < 12; ++k) {
         const int o = hs_dy(k) * W + hs_dx(k);
-        d[k] = ps[2 * W + 2 + o] - ps[2 * W + 2 - o];
-        if (k < 4) de[k] = ro[W + 2 + o] - ro[W + 2 - o];
+        d[k] = P1(ps[2 * W + 2 + o]) - P1(ps[2 * W + 2 - o]);
+        if (k < 4) de[k] = P1(ro[W + 2 + o]) - P1(ro[W + 2 - o]);
     }
 }
 
@@ -160,33 +163,6 @@ __device__ __forceinline__ int column(int x, int nx)
     if (x < 0) x += nx;
     if (x >= nx) x -= nx;
     return x < 0 || x >= nx ? ((x % nx) + nx) % nx : x;
-}
-
-// Sum of one value per lane over the lanes of a row (a power of two of adjacent
-// lanes in each half-warp); FP32 carried as an error-free (hi, lo) pair.
-template <int PW> __device__ __forceinline__ double row_sum(float v)
-{
-    float hi = v, lo = 0.f;
-    auto add = [&](int o) {
-        const float h2 = __shfl_xor_sync(0xffffffffu, hi, o);
-        const float l2 = __shfl_xor_sync(0xffffffffu, lo, o);
-        const float sum = __fadd_rn(hi, h2);
-        const float bp = __fsub_rn(sum, hi);
-        const float err = __fadd_rn(__fsub_rn(hi, __fsub_rn(sum, bp)), __fsub_rn(h2, bp));
-        hi = sum;
-        lo = __fadd_rn(__fadd_rn(lo, l2), err);
-    };
-    add(16);
-#pragma unroll
-    for (int o = PW / 2; o > 0; o >>= 1) add(o);
-    return (double)hi + (double)lo;
-}
-template <int PW> __device__ __forceinline__ double row_sum(double v)
-{
-    v += __shfl_xor_sync(0xffffffffu, v, 16);
-#pragma unroll
-    for (int o = PW / 2; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-    return v;
 }
 
 constexpr int PATCH_THREADS = 512;  // at most 128 registers
@@ -224,6 +200,7 @@ __global__ void __launch_bounds__(PATCH_THREADS) patch_steps_kernel(const __grid
     const int cell_0 = (int)blockIdx.x / per_cell, rem_0 = (int)blockIdx.x - cell_0 * per_cell;
     const int py_0 = rem_0 / a.npx, px_0 = rem_0 - py_0 * a.npx;
 
+    int slot = 0;  // sampled steps so far
     for (int s = 0; s < a.steps; ++s) {
         const T* const fin = reinterpret_cast<const T*>(a.in[s & 1]);
         T* const fout = reinterpret_cast<T*>(a.out[s & 1]);
@@ -259,7 +236,7 @@ __global__ void __launch_bounds__(PATCH_THREADS) patch_steps_kernel(const __grid
                 const T* const src = fc + (q * 9 * pl_el + yy * pitch);
                 if constexpr (NS == 1) {
 #pragma unroll
-                    for (int i = 0; i < 9; ++i) f[i] = __ldcg(src + (i * pl_el + xa));
+                    for (int i = 0; i < 9; ++i) f[i] = V(__ldcg(src + (i * pl_el + xa)));
                 } else if (xb == xa + 1 && (xa & 1) == 0) {
 #pragma unroll
                     for (int i = 0; i < 9; ++i) f[i] = ld_pair(src + (i * pl_el + xa));
@@ -310,7 +287,7 @@ __global__ void __launch_bounds__(PATCH_THREADS) patch_steps_kernel(const __grid
             // ---- collide the pair (the tiled kernel's arithmetic)
             const bool act_a = x < nx && y < ny, act_b = NS == 2 && x + 1 < nx && y < ny;
             const C tau_s = sp ? pg.tau_b : pg.tau, omega_s = sp ? pg.omega_b : pg.omega;
-            const V ga = V(sp ? pg.g1[1] : pg.g1[0]), gr = V(sp ? pg.g2[1] : pg.g2[0]), gx = V(pg.gab_over_rho0);
+            const Couplings<V> cp(pg, sp);
             const V tau2 = V(tau_s), ntau2 = V(-tau_s), omega2 = V(omega_s), mix2 = V(sp ? pg.mix[1] : pg.mix[0]);
             const C rho_bar = sp ? pg.rho_bar[1] : pg.rho_bar[0];
             const bool one_time = pg.mix[0] == C(1);
@@ -319,7 +296,7 @@ __global__ void __launch_bounds__(PATCH_THREADS) patch_steps_kernel(const __grid
             lane_window<W>(psi_s + sp * SS + row * W + NS * pl, rho_s_ + (1 - sp) * SS + (row + 1) * W + NS * pl, dps, dro,
                            &psi, &rho_p);
             const V rho_s = *reinterpret_cast<const V*>(rho_s_ + sp * SS + (row + 2) * W + NS * pl + 2);
-            const Sums<V> sm = stencil_sums<V>(dps, dro);
+            const Pull<V> pu = cp.pull(dps, dro);
             const V jx_s = mom_x<V>(f), jy_s = mom_y<V>(f);
             const V jx_p = from_partner(jx_s), jy_p = from_partner(jy_s);
             V jwx = vfma(mix2, jx_p, jx_s), jwy = vfma(mix2, jy_p, jy_s);
@@ -334,30 +311,30 @@ __global__ void __launch_bounds__(PATCH_THREADS) patch_steps_kernel(const __grid
             const V rho_t = rho_s + rho_p;
             V ax = V(fx_body) * inv_rho;
             if (!one_time && fx_body != C(0)) ax = V(fx_body) * lane_rcp(rho_t);
-            bad |= (act_a && !(first(rho_t) > C(0) && first(rho_t) <= std::numeric_limits<C>::max())) ||
-                   (act_b && !(second(rho_t) > C(0) && second(rho_t) <= std::numeric_limits<C>::max()));
-            V fs[9], Fx, Fy;
+            bad |= (act_a && !density_ok(first(rho_t))) ||
+                   (act_b && !density_ok(second(rho_t)));
+            V fs[9], Fx;
             if constexpr (MRT) {
                 V mh[4];
 #pragma unroll
                 for (int q = 0; q < 4; ++q) mh[q] = V(sp ? pg.mrt_h[1][q] : pg.mrt_h[0][q]);
                 if constexpr (Store<T>::shifted)
-                    collide_species_shifted<V, false, true>(f, rho_s, V(rho_bar), psi, ux, uy, ax, sm, ga, gr, gx, tau2, ntau2, omega2, fs, &Fx, &Fy, V(scale), mh);
+                    collide_species_shifted<V, false, true>(f, rho_s, V(rho_bar), psi, ux, uy, ax, pu, tau2, ntau2, omega2, fs, &Fx, V(scale), mh);
                 else
-                    collide_species<V, false, true>(f, rho_s, psi, ux, uy, ax, sm, ga, gr, gx, tau2, ntau2,
-                                                    omega2, fs, &Fx, &Fy, mh);
+                    collide_species<V, false, true>(f, rho_s, psi, ux, uy, ax, pu, tau2, ntau2,
+                                                    omega2, fs, &Fx, mh);
             } else if constexpr (Store<T>::shifted) {
                 if (unit_omega)
-                    collide_species_shifted<V, true>(f, rho_s, V(rho_bar), psi, ux, uy, ax, sm, ga, gr, gx, tau2, ntau2, omega2, fs, &Fx, &Fy, V(scale));
+                    collide_species_shifted<V, true>(f, rho_s, V(rho_bar), psi, ux, uy, ax, pu, tau2, ntau2, omega2, fs, &Fx, V(scale));
                 else
-                    collide_species_shifted<V, false>(f, rho_s, V(rho_bar), psi, ux, uy, ax, sm, ga, gr, gx, tau2, ntau2, omega2, fs, &Fx, &Fy, V(scale));
+                    collide_species_shifted<V, false>(f, rho_s, V(rho_bar), psi, ux, uy, ax, pu, tau2, ntau2, omega2, fs, &Fx, V(scale));
             } else {
                 if (unit_omega)
-                    collide_species<V, true>(f, rho_s, psi, ux, uy, ax, sm, ga, gr, gx, tau2, ntau2, omega2, fs,
-                                             &Fx, &Fy);
+                    collide_species<V, true>(f, rho_s, psi, ux, uy, ax, pu, tau2, ntau2, omega2, fs,
+                                             &Fx);
                 else
-                    collide_species<V, false>(f, rho_s, psi, ux, uy, ax, sm, ga, gr, gx, tau2, ntau2, omega2, fs,
-                                              &Fx, &Fy);
+                    collide_species<V, false>(f, rho_s, psi, ux, uy, ax, pu, tau2, ntau2, omega2, fs,
+                                              &Fx);
             }
             Dither dz;
             if constexpr (Store<T>::dithered)
@@ -370,6 +347,12 @@ __global__ void __launch_bounds__(PATCH_THREADS) patch_steps_kernel(const __grid
             const int row3[3] = {(y == 0 ? ny - 1 : y - 1) * pitch, y * pitch, (y == ny - 1 ? 0 : y + 1) * pitch};
             const bool wall_lo = a.bc == 1 && y == 0, wall_hi = a.bc == 1 && y == ny - 1;
             C dpx_site = C(0);
+            // this thread's place in the wall momenta of a sampled step
+            constexpr int DW = PatchLane<T>::DW;
+            const int n_units = (nx + NS - 1) / NS;
+            C* const dp = reinterpret_cast<C*>(a.dp) +
+                          (((long long)(slot * g.n_cells + cell) * 2 + (wall_lo ? 1 : 0)) * 2 + sp) * DW * n_units + x / NS;
+            int link = 0;
             if (x0 > 0 && x0 + BX < nx && y0 + BY <= ny && !(wall_lo || wall_hi)) {
                 // away from the edges in x (uniform over the block): fixed offsets
 #pragma unroll
@@ -377,7 +360,7 @@ __global__ void __launch_bounds__(PATCH_THREADS) patch_steps_kernel(const __grid
                     const int cy = q_cy(i), cx = q_cx(i);
                     T* const q = dst + (i * pl_el + off + row3[cy + 1]);
                     if constexpr (NS == 1) {
-                        q[cx] = fs[i];
+                        q[cx] = first(fs[i]);
                     } else if (cx == 0) {
                         st_pair<T, C>(q, first(fs[i]), second(fs[i]), dz);
                     } else {
@@ -408,6 +391,7 @@ __global__ void __launch_bounds__(PATCH_THREADS) patch_steps_kernel(const __grid
                             st_one<T, C>(q, (ba - sh) * scale, dz);
                             dpx_site += dpa;
                         }
+                        if (NS == 1 && sample) dp[link++ * n_units] = dpa;
                     } else {
                         T* const q = dst + (i * pl_el + off + row3[cy + 1]);
                         if (cx == 0 && act_b) {
@@ -430,13 +414,9 @@ __global__ void __launch_bounds__(PATCH_THREADS) patch_steps_kernel(const __grid
                 const C fx_partner = __shfl_xor_sync(0xffffffffu, sp ? first(Fx) : second(Fx), 16);
                 const C Fx_t = (sp ? second(Fx) : first(Fx)) + fx_partner;
                 const C up = ((sp ? second(jxo) : first(jxo)) + C(0.5) * Fx_t) * (sp ? second(inv_r) : first(inv_r));
-                const double u_sum = row_sum<PW>((sp ? act_b : act_a) ? up : C(0));  // one site: species-A lanes
-                const double w_sum = row_sum<PW>(dpx_site);
-                // the row of a patch belongs to this warp in every step
-                if (sp == 0 && pl == 0 && y < ny) {
-                    a.prof[((long long)cell * a.npx + px) * ny + y] += u_sum;
-                    if (wall_lo || wall_hi) a.wall[((long long)cell * a.npx + px) * 2 + (wall_lo ? 1 : 0)] += w_sum;
-                }
+                if (sp ? act_b : act_a)  // one site per thread: species-A lanes
+                    reinterpret_cast<C*>(a.u)[((long long)(slot * g.n_cells + cell) * ny + y) * nx + x + sp] = up;
+                if (NS == 2 && act_a && (wall_lo || wall_hi)) *dp = dpx_site;
             }
             // every thread is done with shared memory and has stored its pair
             __syncthreads();
@@ -453,8 +433,61 @@ __global__ void __launch_bounds__(PATCH_THREADS) patch_steps_kernel(const __grid
                 ++cell;
             }
         }
+        slot += sample ? 1 : 0;
     }
     if (__syncthreads_or(bad) && t == 0) atomicOr(a.err, ERR_NONFINITE);
+}
+
+// Adds the sampled steps of a launch to the time sums, in the order of the tiled
+// kernel with TX = 32 NW columns and its accumulation (so the sums are the same
+// bit for bit): per step the 32-column groups one after another, then the step.
+// One warp per row of a cell.
+template <class C, int NS, int DW, int NW>
+__global__ void __launch_bounds__(128) patch_finish_kernel(const C* __restrict__ u, const C* __restrict__ dp, int samples,
+                                                           int nx, int ny, int n_cells, int bc,
+                                                           double* __restrict__ acc_prof, double* __restrict__ acc_wall)
+{
+    const int w = blockIdx.x * 4 + (threadIdx.x >> 5), lane = threadIdx.x & 31;
+    if (w >= n_cells * ny) return;
+    const int cell = w / ny, y = w - cell * ny, groups = (nx + 31) / 32, n_units = (nx + NS - 1) / NS;
+    constexpr int SEG = 32 / NW;
+    double acc = acc_prof[w];
+    for (int k = 0; k < samples; ++k) {
+        const C* row = u + ((long long)(k * n_cells + cell) * ny + y) * nx;
+        double sum = 0.0;
+        for (int b0 = 0; b0 < groups; b0 += NW) {
+            const double part = group_sum<NW>(lane, [&](int q) {
+                const int x = b0 * 32 + lane * NW + q;
+                return x < nx ? row[x] : C(0);
+            });
+#pragma unroll
+            for (int m = 0; m < NW; ++m)
+                if (b0 + m < groups) sum += __shfl_sync(0xffffffffu, part, m * SEG);
+        }
+        acc += sum;
+    }
+    if (lane == 0) acc_prof[w] = acc;
+    if (bc != 1 || (y != 0 && y != ny - 1)) return;
+    const int wall = y == 0 ? 1 : 0, sp = lane >> 4;
+    acc = acc_wall[cell * 2 + wall];
+    for (int k = 0; k < samples; ++k) {
+        const C* d = dp + (((long long)(k * n_cells + cell) * 2 + wall) * 2 + sp) * DW * n_units;
+        double sum = 0.0;
+        for (int b = 0; b < groups; ++b) {
+            const int x = b * 32 + 2 * (lane & 15);
+            C v = C(0);
+            if constexpr (NS == 2) {
+                if (x < nx) v = d[x / 2];
+            } else {
+#pragma unroll
+                for (int i = 0; i < DW; ++i)
+                    v += (x < nx ? d[i * n_units + x] : C(0)) + (x + 1 < nx ? d[i * n_units + x + 1] : C(0));
+            }
+            sum += __shfl_sync(0xffffffffu, warp_sum_compensated2(v, C(0)), 0);
+        }
+        acc += sum;
+    }
+    if (lane == 0) acc_wall[cell * 2 + wall] = acc;
 }
 
 // ------------------------------------------------------------- host side --
@@ -465,8 +498,10 @@ struct PatchPlan {
     int grid[2];  // resident blocks: BGK, MRT
     size_t smem;
     int mrt = 0;
-    unsigned* flags = nullptr;
-    double *prof = nullptr, *wall = nullptr;
+    int slots;  // sampled steps a launch may hold
+    void* mem = nullptr;  // one allocation: the sampled steps' values and the flags
+    void *u, *dp;
+    unsigned* flags;
 };
 
 template <class T, int PW> static const void* patch_kernel(bool mrt)
@@ -487,9 +522,7 @@ static const void* patch_kernel(int prec, int pw, bool mrt)
 void patch_destroy(PatchPlan* p)
 {
     if (!p) return;
-    cudaFree(p->flags);
-    cudaFree(p->prof);
-    cudaFree(p->wall);
+    cudaFree(p->mem);
     delete p;
 }
 
@@ -498,7 +531,8 @@ void patch_destroy(PatchPlan* p)
 // 9, 12 and 16 rows and 8- and 16-column patches on 64^2 .. 512^2 cells: at 256^2
 // FP32 5.98 us per step against 9.4 (32 x 4) and 10.1 (16 x 8).  Below 10240 sites
 // FP64 takes 8 x 4 patches: 64^2 then has 128 of them, one for nearly every SM
-// (12.3 us against 19.6), whose FP64 pipes are the bound.
+// (12.3 us against 19.6), whose FP64 pipes are the bound; above, 16 columns by the
+// 5 to 8 rows that spread best (256^2: 7 rows 44.8 us, 8 rows 49.6).
 PatchPlan* patch_create(const Geom& g, int prec, int bc)
 {
     if (18 * g.plane >= (1LL << 31)) return nullptr;  // 32-bit element offsets inside a cell
@@ -508,7 +542,17 @@ PatchPlan* patch_create(const Geom& g, int prec, int bc)
     cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, dev);
     if (!coop) return nullptr;
     const bool few = prec == LB_FP64 && (long long)g.nx * g.ny * g.n_cells <= 10240;
-    const int pw = few ? 8 : 16, by = few ? 4 : 8;
+    const int pw = few ? 8 : 16;
+    int by = few ? 4 : 8;
+    if (prec == LB_FP64 && !few) {
+        // bound by the SMs' FP64 pipes: the height that gives the fullest SM least to do
+        auto load = [&](int h) {
+            const long long n = (long long)((g.nx + 15) / 16) * ((g.ny + h - 1) / h) * g.n_cells;
+            return ((n + sms - 1) / sms) * (h + 3);  // rows of a patch, and its halo's densities
+        };
+        for (int h = 7; h >= 5; --h)
+            if (load(h) < load(by)) by = h;
+    }
     PatchPlan* p = new PatchPlan();
     p->g = g;
     p->prec = prec;
@@ -533,22 +577,51 @@ PatchPlan* patch_create(const Geom& g, int prec, int bc)
         }
         p->grid[m] = (int)std::min<long long>(n, (long long)occ * sms);
     }
-    if (cudaMalloc(&p->flags, sizeof(unsigned) * n) != cudaSuccess ||
-        cudaMalloc(&p->prof, sizeof(double) * g.n_cells * p->npx * g.ny) != cudaSuccess ||
-        cudaMalloc(&p->wall, sizeof(double) * g.n_cells * p->npx * 2) != cudaSuccess) {
+    // up to 32 sampled steps per launch in 4 MB (at least one)
+    const size_t cb = prec == LB_FP64 ? 8 : 4, u_bytes = cb * g.n_cells * g.ny * g.nx;
+    const size_t dp_bytes = cb * g.n_cells * 4 * (prec == LB_FP64 ? 3 * (size_t)g.nx : (size_t)(g.nx + 1) / 2);
+    p->slots = (int)std::max<size_t>(1, std::min<size_t>(32, (4u << 20) / u_bytes));
+    const size_t u_all = (u_bytes * p->slots + 15) / 16 * 16, dp_all = (dp_bytes * p->slots + 15) / 16 * 16;
+    if (cudaMalloc(&p->mem, u_all + dp_all + sizeof(unsigned) * n) != cudaSuccess) {
         cudaGetLastError();
         patch_destroy(p);
         return nullptr;
     }
+    p->u = p->mem;
+    p->dp = (char*)p->mem + u_all;
+    p->flags = (unsigned*)((char*)p->mem + u_all + dp_all);
     return p;
 }
 
+int patch_max_samples(const PatchPlan* p) { return p->slots; }
+
 void patch_set_collision(PatchPlan* p, int collision) { p->mrt = collision == TILED_MRT; }
 
-cudaError_t launch_patch_steps(PatchPlan* p, void* src, void* dst, int steps, int first, int every, bool swap,
+template <class C, int NS, int DW>
+static void launch_patch_finish(const PatchPlan* p, int samples, int tile_x, double* acc_prof, double* acc_wall,
+                                cudaStream_t st)
+{
+    const Geom& g = p->g;
+    const dim3 grid((g.n_cells * g.ny + 3) / 4);
+    auto go = [&](auto kernel) {
+        kernel<<<grid, 128, 0, st>>>((const C*)p->u, (const C*)p->dp, samples, g.nx, g.ny, g.n_cells, p->bc, acc_prof,
+                                     acc_wall);
+    };
+    switch (tile_x) {
+    case 64: return go(patch_finish_kernel<C, NS, DW, 2>);
+    case 128: return go(patch_finish_kernel<C, NS, DW, 4>);
+    case 256: return go(patch_finish_kernel<C, NS, DW, 8>);
+    default: return go(patch_finish_kernel<C, NS, DW, 1>);
+    }
+}
+
+cudaError_t launch_patch_steps(PatchPlan* p, void* src, void* dst, int steps, int first, int every, bool swap, int tile_x,
                                const CellDev* cells, double* acc_prof, double* acc_wall, unsigned* err,
                                cudaStream_t st, int* n_launches)
 {
+    const int samples = first < 0 ? 0 : (steps - 1 - first) / every + 1;
+    cudaError_t e = cudaSuccess;
+    if (samples > p->slots) return cudaErrorInvalidValue;
     PatchArgs a{};
     a.in[0] = src;
     a.out[0] = dst;
@@ -562,28 +635,25 @@ cudaError_t launch_patch_steps(PatchPlan* p, void* src, void* dst, int steps, in
     a.first = first;
     a.every = every > 0 ? every : 1;
     a.cells = cells;
-    a.prof = p->prof;
-    a.wall = p->wall;
+    a.u = p->u;
+    a.dp = p->dp;
     a.err = err;
     a.flags = p->flags;
-    const Geom& g = p->g;
-    cudaError_t e = cudaSuccess;
-    if (steps > 1) e = cudaMemsetAsync(p->flags, 0, sizeof(unsigned) * g.n_cells * p->npx * p->npy, st);
-    if (e == cudaSuccess && first >= 0) {
-        e = cudaMemsetAsync(p->prof, 0, sizeof(double) * g.n_cells * p->npx * g.ny, st);
-        if (e == cudaSuccess) e = cudaMemsetAsync(p->wall, 0, sizeof(double) * g.n_cells * p->npx * 2, st);
-    }
+    if (steps > 1) e = cudaMemsetAsync(p->flags, 0, sizeof(unsigned) * p->g.n_cells * p->npx * p->npy, st);
     if (e != cudaSuccess) return e;
     void* args[] = {(void*)&a};
     e = cudaLaunchCooperativeKernel(patch_kernel(p->prec, p->pw, p->mrt != 0), dim3(p->grid[p->mrt]),
                                     dim3(32 * p->by / (16 / p->pw)), args, p->smem, st);
     if (e != cudaSuccess) return e;
     *n_launches += 1;
-    if (first >= 0) {
-        e = launch_accumulate(p->prof, p->wall, p->npx, g.ny, p->bc, g.n_cells, acc_prof, acc_wall, st);
+    if (samples > 0) {
+        if (p->prec == LB_FP64)
+            launch_patch_finish<double, 1, 3>(p, samples, tile_x, acc_prof, acc_wall, st);
+        else
+            launch_patch_finish<float, 2, 1>(p, samples, tile_x, acc_prof, acc_wall, st);
         *n_launches += 1;
     }
-    return e;
+    return cudaGetLastError();
 }
 
 }  // namespace lbhb

@@ -120,36 +120,7 @@ __device__ __noinline__ void profile_row_sums(const C* ub, int lane, double* __r
 {
     constexpr int NW = TX / 32, SEG = 32 / NW;
     const int grp = lane / SEG, t = lane % SEG;
-    double part;
-    if constexpr (sizeof(C) == 4) {
-        float hi = ub[grp * 32 + t * NW], lo = 0.f;
-#pragma unroll
-        for (int q = 1; q < NW; ++q) {
-            const float v = ub[grp * 32 + t * NW + q];
-            const float sum = __fadd_rn(hi, v);
-            const float bp = __fsub_rn(sum, hi);
-            lo = __fadd_rn(lo, __fadd_rn(__fsub_rn(hi, __fsub_rn(sum, bp)), __fsub_rn(v, bp)));
-            hi = sum;
-        }
-#pragma unroll
-        for (int o = SEG / 2; o > 0; o >>= 1) {
-            const float h2 = __shfl_down_sync(0xffffffffu, hi, o, SEG);
-            const float l2 = __shfl_down_sync(0xffffffffu, lo, o, SEG);
-            const float sum = __fadd_rn(hi, h2);
-            const float bp = __fsub_rn(sum, hi);
-            const float err = __fadd_rn(__fsub_rn(hi, __fsub_rn(sum, bp)), __fsub_rn(h2, bp));
-            hi = sum;
-            lo = __fadd_rn(__fadd_rn(lo, l2), err);
-        }
-        part = (double)hi + (double)lo;
-    } else {
-        double v = 0.0;
-#pragma unroll
-        for (int q = 0; q < NW; ++q) v += ub[grp * 32 + t * NW + q];
-#pragma unroll
-        for (int o = SEG / 2; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o, SEG);
-        part = v;
-    }
+    const double part = group_sum<NW>(lane, [&](int q) { return ub[grp * 32 + t * NW + q]; });
     const int nbx = (nx + 31) / 32;  // 32-column groups of the lattice; a narrow last strip has fewer
     if (t == 0 && (x0 >> 5) + grp < nbx) prof_part[((long long)cell * nbx + (x0 >> 5) + grp) * nrows + row] = part;
 }
@@ -281,7 +252,6 @@ __global__ void __launch_bounds__(tiled_threads(TX),
         ParamSet<C> p;
         p.rho0 = pg.rho0;
         p.inv_rho0 = pg.inv_rho0;
-        p.gab_over_rho0 = pg.gab_over_rho0;
         p.u_wall = pg.u_wall;
         p.f0 = pg.f0;
         p.two_over_ny = pg.two_over_ny;
@@ -299,7 +269,7 @@ __global__ void __launch_bounds__(tiled_threads(TX),
 #pragma unroll
         for (int q = 0; q < 4; ++q) mh[q] = V(MRT ? (sp ? pg.mrt_h[1][q] : pg.mrt_h[0][q]) : C(0));
         // the same values as lane pairs
-        const V ga = V(sp ? pg.g1[1] : pg.g1[0]), gr = V(sp ? pg.g2[1] : pg.g2[0]), gx = V(p.gab_over_rho0);
+        const Couplings<V> cp(pg, sp);
         const V tau2 = V(tau_s), ntau2 = V(-tau_s), omega2 = V(omega_s), mix2 = V(mix);
         const V rho0_2 = V(p.rho0), inv_rho0_2 = V(p.inv_rho0);
         const C rho_bar = sp ? pg.rho_bar[1] : pg.rho_bar[0];
@@ -431,7 +401,7 @@ __global__ void __launch_bounds__(tiled_threads(TX),
             // pair differences d_q = psi(r + c_q) - psi(r - c_q) of both sites
             V dps[12], dro[4];
             window_diffs(v, e, dps, dro);
-            const Sums<V> sm = stencil_sums<V>(dps, dro);
+            const Pull<V> pu = cp.pull(dps, dro);
             const V jx_s = mom_x<V>(f), jy_s = mom_y<V>(f);
             const V jx_p(__shfl_xor_sync(0xffffffffu, jx_s.a(), 16), __shfl_xor_sync(0xffffffffu, jx_s.b(), 16));
             const V jy_p(__shfl_xor_sync(0xffffffffu, jy_s.a(), 16), __shfl_xor_sync(0xffffffffu, jy_s.b(), 16));
@@ -459,29 +429,25 @@ __global__ void __launch_bounds__(tiled_threads(TX),
             if (body_raw) ax = V(fx_body) * lane_rcp(rho_t);
             // watchdog: a non-finite or non-positive total density anywhere in the
             // item is reported through the error word when the item ends
-            if (act) bad |= !(rho_t.a() > C(0) && rho_t.a() <= std::numeric_limits<C>::max() && rho_t.b() > C(0) &&
-                              rho_t.b() <= std::numeric_limits<C>::max());
-            V fs[9], Fx, Fy;
+            if (act) bad |= !(density_ok(rho_t.a()) && density_ok(rho_t.b()));
+            V fs[9], Fx;
             if constexpr (MRT && Store<T>::shifted) {
-                collide_species_shifted<V, false, true>(f, rho_s, rho_bar2, v[2][1], ux, uy, ax, sm, ga, gr, gx,
-                                                        tau2, ntau2, omega2, fs, &Fx, &Fy, V(scale), mh);
+                collide_species_shifted<V, false, true>(f, rho_s, rho_bar2, v[2][1], ux, uy, ax, pu, tau2, ntau2, omega2, fs, &Fx, V(scale), mh);
             } else if constexpr (MRT) {
-                collide_species<V, false, true>(f, rho_s, v[2][1], ux, uy, ax, sm, ga, gr, gx, tau2, ntau2, omega2,
-                                                fs, &Fx, &Fy, mh);
+                collide_species<V, false, true>(f, rho_s, v[2][1], ux, uy, ax, pu, tau2, ntau2, omega2,
+                                                fs, &Fx, mh);
             } else if constexpr (Store<T>::shifted) {
                 if (unit_omega)
-                    collide_species_shifted<V, true>(f, rho_s, rho_bar2, v[2][1], ux, uy, ax, sm, ga, gr, gx, tau2,
-                                                     ntau2, omega2, fs, &Fx, &Fy, V(scale));
+                    collide_species_shifted<V, true>(f, rho_s, rho_bar2, v[2][1], ux, uy, ax, pu, tau2, ntau2, omega2, fs, &Fx, V(scale));
                 else
-                    collide_species_shifted<V, false>(f, rho_s, rho_bar2, v[2][1], ux, uy, ax, sm, ga, gr, gx, tau2,
-                                                      ntau2, omega2, fs, &Fx, &Fy, V(scale));
+                    collide_species_shifted<V, false>(f, rho_s, rho_bar2, v[2][1], ux, uy, ax, pu, tau2, ntau2, omega2, fs, &Fx, V(scale));
             } else {
                 if (unit_omega)
-                    collide_species<V, true>(f, rho_s, v[2][1], ux, uy, ax, sm, ga, gr, gx, tau2, ntau2, omega2, fs,
-                                             &Fx, &Fy);
+                    collide_species<V, true>(f, rho_s, v[2][1], ux, uy, ax, pu, tau2, ntau2, omega2, fs,
+                                             &Fx);
                 else
-                    collide_species<V, false>(f, rho_s, v[2][1], ux, uy, ax, sm, ga, gr, gx, tau2, ntau2, omega2, fs,
-                                              &Fx, &Fy);
+                    collide_species<V, false>(f, rho_s, v[2][1], ux, uy, ax, pu, tau2, ntau2, omega2, fs,
+                                              &Fx);
             }
 
             // stochastic rounding: one stream per thread and row, seeded from the
