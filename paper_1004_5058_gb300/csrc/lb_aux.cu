@@ -8,7 +8,7 @@ namespace lbhb {
 // evaluated in the compute type of the storage (FP32 for FP32 and FP16 storage:
 // the FP64 pipe would make this initialisation ten times slower than its
 // memory traffic), the +-c pairs together as in the collision.
-// src: device float64 [cell][4][ny][nx] = rho_A, rho_B, u_x, u_y.
+// src: device float64 [4][cell][ny][nx] = rho_A, rho_B, u_x, u_y.
 template <class T>
 __global__ void equilibrium_kernel(const double* __restrict__ src, T* __restrict__ f, Geom g,
                                    const CellDev* __restrict__ cells)
@@ -16,8 +16,8 @@ __global__ void equilibrium_kernel(const double* __restrict__ src, T* __restrict
     using C = typename Store<T>::C;
     const int x = blockIdx.x * blockDim.x + threadIdx.x, y = blockIdx.y, cell = blockIdx.z;
     if (x >= g.nx) return;
-    const long long n = (long long)g.nx * g.ny, k = (long long)y * g.nx + x;
-    const double* s0 = src + (long long)cell * 4 * n;
+    const long long n = (long long)g.nx * g.ny * g.n_cells, k = ((long long)cell * g.ny + y) * g.nx + x;
+    const double* s0 = src;
     const C ux = C(s0[2 * n + k]), uy = C(s0[3 * n + k]);
     const C base = C(1) - C(1.5) * (ux * ux + uy * uy);
     const C cu[4] = {ux, uy, ux + uy, uy - ux};  // c.u for i = 1, 2, 5, 6
@@ -66,7 +66,7 @@ __global__ void import_kernel(const double* __restrict__ src, T* __restrict__ f,
 }
 
 // Per-site rho_A, rho_B, and the paper's u = j / rho into dense float64
-// [cell][4][ny][nx]; flags non-finite or non-positive densities.
+// [4][cell][ny][nx] (so that each field is one contiguous copy to the host); flags non-finite or non-positive densities.
 template <class T>
 __global__ void fields_kernel(const T* __restrict__ f, double* __restrict__ dst, Geom g,
                               const CellDev* __restrict__ cells, unsigned* __restrict__ err)
@@ -87,8 +87,8 @@ __global__ void fields_kernel(const T* __restrict__ f, double* __restrict__ dst,
         jx += (double)((v[1] - v[3]) + (v[5] - v[7]) + (v[8] - v[6]));
         jy += (double)((v[2] - v[4]) + (v[5] - v[7]) + (v[6] - v[8]));
     }
-    const long long n = (long long)g.nx * g.ny, k = (long long)y * g.nx + x;
-    double* d = dst + (long long)cell * 4 * n;
+    const long long n = (long long)g.nx * g.ny * g.n_cells, k = ((long long)cell * g.ny + y) * g.nx + x;
+    double* d = dst;
     const double rt = rho[0] + rho[1];
     d[k] = rho[0];
     d[n + k] = rho[1];
