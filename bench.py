@@ -124,7 +124,7 @@ def source_digest():
     editing a comment does not orphan the committed DRAM counters)."""
     import re
     h = hashlib.sha256()
-    for f in ("lb_tiled.cu", "lb_common.cuh", "tma.cuh"):
+    for f in ("lb_tiled.cuh", "lb_common.cuh", "lb_pair.cuh", "tma.cuh"):
         with open(os.path.join(ROOT, "paper_1004_5058_gb300", "csrc", f)) as fh:
             src = fh.read()
         src = re.sub(r"/\*.*?\*/", " ", src, flags=re.S)

@@ -67,7 +67,10 @@ struct lb_handle {
     lb_kernel kernel = LB_KERNEL_GENERIC;
     int tile_x = 0, tile_y = 0;
     TiledPlan* plan = nullptr;
-    PatchPlan* patch = nullptr;  // small lattices under LB_KERNEL_AUTO: lb_step runs this one
+    // under LB_KERNEL_AUTO (at most one of them): small lattices, which lb_step runs many
+    // steps at a time; large ones of a width lb_set_kernel refuses to the tiled kernel
+    PatchPlan* patch = nullptr;
+    TiledPlan* any_width = nullptr;
     long long launches = 0;
     int inject = 0;  // lb_test_inject: 1 = stalled row copy, 2 = failed launch (next lb_step)
     std::string last_error;
@@ -114,6 +117,7 @@ static void release(lb_handle* h)
     free_graphs(h);
     if (h->plan) tiled_destroy(h->plan);
     patch_destroy(h->patch);
+    if (h->any_width) tiled_destroy(h->any_width);
     cudaFree(h->f[0]);
     cudaFree(h->f[1]);
     cudaFree(h->aux);
@@ -271,10 +275,12 @@ static lb_status select_by_shape(lb_handle* h)
     return select_kernel(h, LB_KERNEL_GENERIC, 0, 0);
 }
 
-static void drop_patch(lb_handle* h)
+static void drop_auto(lb_handle* h)
 {
     patch_destroy(h->patch);
     h->patch = nullptr;
+    if (h->any_width) tiled_destroy(h->any_width);
+    h->any_width = nullptr;
 }
 
 // Under LB_KERNEL_AUTO a small lattice steps through the patch kernel.  us per
@@ -286,19 +292,31 @@ static void drop_patch(lb_handle* h)
 // The tiled kernel's time hardly depends on the size up to 2^17 sites (its rows
 // are a serial chain), the patch kernel's grows with it; they meet near there, and
 // with the FP64 generic pair, which spreads over the chip as well, near 2^15.
-static void select_patch(lb_handle* h)
+// Larger FP32 and FP16 lattices whose width lb_set_kernel refuses to the tiled
+// kernel run its any-width form instead of the generic pair (us per step, generic
+// / any width: 1021 x 509 FP32 39.5 / 18.8, FP16 44.7 / 22.1; 1021 x 1509 123 / 50;
+// 401 x 399 15.8 / 14.4; 16 cells of 101 x 260 41.5 / 22.0).  FP64 stays with the
+// pair: its pipe bounds both (1021 x 509 293 us).
+static void select_beyond_family(lb_handle* h)
 {
+    if (h->slab) return;
     const long long most = h->kernel == LB_KERNEL_GENERIC && h->prec == LB_FP64 ? 1LL << 15 : 1LL << 17;
-    if (h->slab || (long long)h->n_cells * h->nx * h->ny >= most) return;
-    h->patch = patch_create(h->g, (int)h->prec, h->bc);
-    if (h->patch) patch_set_collision(h->patch, collision_kind(h->cells));
+    if ((long long)h->n_cells * h->nx * h->ny < most) {
+        h->patch = patch_create(h->g, (int)h->prec, h->bc);
+        if (h->patch) patch_set_collision(h->patch, collision_kind(h->cells));
+    } else if (h->kernel == LB_KERNEL_GENERIC) {
+        const int tx = h->nx >= 128 ? 128 : 64;
+        if (tiled_any_supported(h->gbuf, h->elem, tx))
+            h->any_width = tiled_create(h->gbuf, h->rm, (int)h->prec, h->elem, h->bc, h->f[0], h->f[1], tx, 0, true, nullptr);
+        if (h->any_width) tiled_set_collision(h->any_width, collision_kind(h->cells));
+    }
 }
 
 static lb_status select_kernel(lb_handle* h, lb_kernel k, int tx, int ty)
 {
     if (k == LB_KERNEL_AUTO) {
         const lb_status st = select_by_shape(h);
-        if (st == LB_OK) select_patch(h);
+        if (st == LB_OK) select_beyond_family(h);
         return st;
     }
     if (k == LB_KERNEL_GENERIC && h->slab)
@@ -309,7 +327,7 @@ static lb_status select_kernel(lb_handle* h, lb_kernel k, int tx, int ty)
             tiled_destroy(h->plan);
             h->plan = nullptr;
         }
-        drop_patch(h);
+        drop_auto(h);
         h->kernel = LB_KERNEL_GENERIC;
         h->tile_x = 32;
         h->tile_y = 8;
@@ -330,11 +348,11 @@ static lb_status select_kernel(lb_handle* h, lb_kernel k, int tx, int ty)
     if (tiled_partials_nbx(h->g, tx) > h->nbx_alloc)
         return fail(h, LB_ERR_UNSUPPORTED, "lb_set_kernel: tile %d too narrow for the partial buffers", tx);
     const char* msg = nullptr;
-    TiledPlan* p = tiled_create(h->gbuf, h->rm, (int)h->prec, h->elem, h->bc, h->f[0], h->f[1], tx, ty, &msg);
+    TiledPlan* p = tiled_create(h->gbuf, h->rm, (int)h->prec, h->elem, h->bc, h->f[0], h->f[1], tx, ty, false, &msg);
     if (!p) return fail(h, LB_ERR_UNSUPPORTED, "lb_set_kernel: %s", msg ? msg : "tiled plan failed");
     tiled_set_collision(p, collision_kind(h->cells));
     if (h->plan) tiled_destroy(h->plan);
-    drop_patch(h);
+    drop_auto(h);
     h->plan = p;
     h->kernel = LB_KERNEL_TILED;
     tiled_tiles(p, &h->tile_x, &h->tile_y);
@@ -758,18 +776,21 @@ lb_status lb_get_populations(lb_handle* h, double* f)
     return LB_OK;
 }
 
+// The tiled plan that a step runs, or nullptr for the generic pair.
+static TiledPlan* step_plan(const lb_handle* h) { return h->kernel == LB_KERNEL_TILED ? h->plan : h->any_width; }
+
 static cudaError_t enqueue_one_step(lb_handle* h, int src, bool sample, int* nl)
 {
     cudaError_t e = with_type(h, [&](auto* tp) {
         using T = std::remove_pointer_t<decltype(tp)>;
-        if (h->kernel == LB_KERNEL_TILED)
-            return launch_tiled_step<T>(h->plan, src, h->d_cells, sample, h->prof_part, h->wall_part, h->d_err,
+        if (TiledPlan* plan = step_plan(h))
+            return launch_tiled_step<T>(plan, src, h->d_cells, sample, h->prof_part, h->wall_part, h->d_err,
                                         h->stream, nl);
         return launch_generic_step<T>((const T*)h->f[src], (T*)h->f[1 - src], h->g, h->bc, h->d_cells, h->aux,
                                       sample, h->prof_part, h->wall_part, h->d_err, h->stream, nl);
     });
     if (e != cudaSuccess || !sample) return e;
-    const int nbx = h->kernel == LB_KERNEL_TILED ? tiled_partials_nbx(h->g, h->tile_x) : generic_partials_nbx(h->g);
+    const int nbx = step_plan(h) ? tiled_partials_nbx(h->g, h->tile_x) : generic_partials_nbx(h->g);
     *nl += 1;
     return launch_accumulate(h->prof_part, h->wall_part, nbx, h->ny, h->bc, h->n_cells, h->acc_prof, h->acc_wall,
                              h->stream);
@@ -824,7 +845,7 @@ static cudaError_t run_chunk(lb_handle* h, int src, int steps, bool sample_last,
         it = h->graphs.emplace(key, exec).first;
     }
     // count the launches the graph holds
-    int kernels_per_step = h->kernel == LB_KERNEL_TILED ? 1 : 2;
+    int kernels_per_step = step_plan(h) ? 1 : 2;
     *nl += steps * kernels_per_step + (sample_last ? 1 : 0);
     return cudaGraphLaunch(it->second, h->stream);
 }
@@ -1135,7 +1156,7 @@ lb_status lb_autotune(lb_handle* h, const char* cache_path)
     }
     // candidates: generic, and every supported tile
     std::vector<std::tuple<int, int, int>> cand;
-    cand.emplace_back((int)LB_KERNEL_AUTO, 0, 0);  // the patch kernel, where it serves the lattice
+    cand.emplace_back((int)LB_KERNEL_AUTO, 0, 0);  // select_beyond_family, where it serves the lattice
     cand.emplace_back((int)LB_KERNEL_GENERIC, 0, 0);
     const int txs[] = {32, 64, 128, 256};
     const int tys[] = {0, 16, 32, 64};  // 0: segment height from the fill model
@@ -1150,8 +1171,8 @@ lb_status lb_autotune(lb_handle* h, const char* cache_path)
     const int reps = 6, patch_reps = 64;  // the patch kernel takes many steps per launch
     for (auto& c : cand) {
         if (select_kernel(h, (lb_kernel)std::get<0>(c), std::get<1>(c), std::get<2>(c)) != LB_OK) continue;
-        const bool patch = std::get<0>(c) == LB_KERNEL_AUTO;
-        if (patch && !h->patch) continue;
+        const bool patch = std::get<0>(c) == LB_KERNEL_AUTO && h->patch;
+        if (std::get<0>(c) == LB_KERNEL_AUTO && !h->patch && !h->any_width) continue;
         int nl = 0;
         // trial steps read the current buffer and write the other one, without
         // swapping, so the state is unchanged
@@ -1366,6 +1387,7 @@ lb_status lb_load(lb_handle* h, const char* path)
     h->cells = cells;
     if (h->plan) tiled_set_collision(h->plan, collision_kind(h->cells));
     if (h->patch) patch_set_collision(h->patch, collision_kind(h->cells));
+    if (h->any_width) tiled_set_collision(h->any_width, collision_kind(h->cells));
     free_graphs(h);  // captured launches may name the other kernel family
     h->cur = 0;
     h->t = hd.t;

@@ -15,13 +15,16 @@ int generic_partials_nbx(const Geom& g);
 // tiled family (lb_tiled.cu)
 struct TiledPlan;  // opaque per-handle state of the tiled kernel
 bool tiled_supported(const Geom& g, int elem_bytes, int tile_x, int tile_y);
+// Any width of at least tile_x (64 or 128) columns, odd ones too (whole cells, FP32
+// and FP16 storage): LB_KERNEL_AUTO runs it where tiled_supported says no.
+bool tiled_any_supported(const Geom& g, int elem_bytes, int tile_x);
 int tiled_partials_nbx(const Geom& g, int tile_x);
 // Creates the plan (tensor maps for both ping-pong buffers).  Returns nullptr
 // and sets *err_msg if the shape/tile is not supported or encoding failed.
 // g: the whole population buffer; rm: the rows a step updates (a whole cell, or
 // the own rows of a slab between its ghost rows).
 TiledPlan* tiled_create(const Geom& g, const RowMap& rm, int prec, int elem_bytes, int bc, void* f0, void* f1,
-                        int tile_x, int tile_y, const char** err_msg);
+                        int tile_x, int tile_y, bool any, const char** err_msg);
 void tiled_destroy(TiledPlan* p);
 template <class T>
 cudaError_t launch_tiled_step(TiledPlan* p, int src_buf, const CellDev* cells, bool sample, double* prof_part,
