@@ -68,7 +68,7 @@ typedef enum { LB_BC_PERIODIC = 0, LB_BC_COUETTE = 1 } lb_bc;
 typedef enum { LB_FP32 = 0, LB_FP16_SHIFTED = 1, LB_FP64 = 2, LB_FP16_SHIFTED_SR = 3 } lb_precision;
 
 /* Kernel family: AUTO picks TILED when the shape allows it, else GENERIC.  Under
- * AUTO lb_step advances a small lattice (below 2^17 sites over all cells) with a kernel
+ * AUTO lb_step advances a small lattice (below 2^16 sites over all cells, FP64 2^17) with a kernel
  * that takes many steps per launch; the family AUTO picked then serves steps
  * inside a capture of the caller's and is what lb_get_kernel reports. */
 typedef enum { LB_KERNEL_AUTO = 0, LB_KERNEL_GENERIC = 1, LB_KERNEL_TILED = 2 } lb_kernel;

@@ -264,12 +264,13 @@ static lb_status select_kernel(lb_handle* h, lb_kernel k, int tx, int ty);
 // The kernel family and tile of LB_KERNEL_AUTO.
 static lb_status select_by_shape(lb_handle* h)
 {
-    // the widest tile that divides nx, else the widest that fits (a narrower
-    // last strip), else the generic kernel
+    // 128 or 64 columns where they divide nx, else the widest tile that fits (a
+    // narrower last strip), else the generic kernel.  32 columns are left to lattices
+    // narrower than 64: us per step 352^2 FP32 9.8 (32) / 8.4 (128), 200^2 FP64 106 / 46
     const int txs[] = {128, 64, 32};
     for (int pass = 0; pass < 2; ++pass)
         for (int c : txs)
-            if ((pass == 1 || h->nx % c == 0) && tiled_supported(h->gbuf, h->elem, c, 0) &&
+            if ((pass == 1 || (c > 32 && h->nx % c == 0)) && tiled_supported(h->gbuf, h->elem, c, 0) &&
                 select_kernel(h, LB_KERNEL_TILED, c, 0) == LB_OK)
                 return LB_OK;
     return select_kernel(h, LB_KERNEL_GENERIC, 0, 0);
@@ -284,14 +285,13 @@ static void drop_auto(lb_handle* h)
 }
 
 // Under LB_KERNEL_AUTO a small lattice steps through the patch kernel.  us per
-// step, the kernel of select_by_shape against the patch kernel (one cell):
-//   FP32  64^2 9.3 / 3.2, 128^2 10.4 / 3.4, 256^2 10.4 / 6.0, 384^2 10.5 / 9.7, 512^2 12.3 / 16.1;
-//   FP64  64^2 84 / 11, 128^2 97 / 14, 256^2 97 / 45, 320^2 100 / 75, 360^2 102 / 100;
-//   37 x 23 (generic pair) FP32 5.5 / 3.6, 301 x 243 FP32 10.1 / 9.0;
-//   101 x 83 (generic pair) FP64 24 / 12, 201 x 163 FP64 24.4 / 26.5.
-// The tiled kernel's time hardly depends on the size up to 2^17 sites (its rows
-// are a serial chain), the patch kernel's grows with it; they meet near there, and
-// with the FP64 generic pair, which spreads over the chip as well, near 2^15.
+// step, the kernel of select_by_shape against the patch kernel:
+//   FP32  64^2 6.0 / 3.2, 192^2 5.8 / 3.7, 256^2 6.5 / 6.6, 288^2 7.2 / 9.1; cells of
+//         64^2: 16 6.5 / 5.5, 24 7.5 / 8.2;  37 x 23 (generic pair) 5.5 / 3.6;
+//   FP64  64^2 84 / 11, 128^2 97 / 14, 256^2 56 / 45, 320^2 88 / 75, 352^2 99 / 100;
+//         101 x 83 (generic pair) 24 / 12, 201 x 163 (generic pair) 24.4 / 26.5.
+// The patch kernel's time grows with the sites each SM holds; they meet near 2^16
+// sites in FP32 and FP16, 2^17 in FP64, and 2^15 with the FP64 generic pair.
 // Larger FP32 and FP16 lattices whose width lb_set_kernel refuses to the tiled
 // kernel run its any-width form instead of the generic pair (us per step, generic
 // / any width: 1021 x 509 FP32 39.5 / 18.8, FP16 44.7 / 22.1; 1021 x 1509 123 / 50;
@@ -300,7 +300,7 @@ static void drop_auto(lb_handle* h)
 static void select_beyond_family(lb_handle* h)
 {
     if (h->slab) return;
-    const long long most = h->kernel == LB_KERNEL_GENERIC && h->prec == LB_FP64 ? 1LL << 15 : 1LL << 17;
+    const long long most = h->prec != LB_FP64 ? 1LL << 16 : h->kernel == LB_KERNEL_GENERIC ? 1LL << 15 : 1LL << 17;
     if ((long long)h->n_cells * h->nx * h->ny < most) {
         h->patch = patch_create(h->g, (int)h->prec, h->bc);
         if (h->patch) patch_set_collision(h->patch, collision_kind(h->cells));

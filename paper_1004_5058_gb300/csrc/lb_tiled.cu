@@ -72,22 +72,35 @@ static size_t smem_bytes(int tx, int elem, int depth)
 }
 static_assert(tiled_smem_bytes(128, 4) == 74032, "shared memory of the FP32 128-column tile");
 
-// Segment height from a fill model: work items = strips x segments x cells run
-// on `slots` persistent CTAs, each item costing about (rows + 6) row-times
-// (4 halo rows plus pipeline effects); pick the height with the least
-// rounds x cost, so the last round of items is not mostly empty.  A narrower last
-// strip counts as a strip: leaving it out gave 1000 x 1000 FP32 16-row segments in
-// two rounds, 38.4 us per step, where 18 rows take one, 30.0 us.
-static int pick_segment_rows(const Geom& g, int nrows, int tile_x, long long slots)
+// Segment height from a model of the time of a launch: work items = strips x
+// segments x cells; an item walks its rows, four halo rows and about 1.5 row-times
+// of start-up one after another, and a row takes longer the more column warps share
+// the SM.  us per row measured on 384^2 .. 1024^2 FP32 cells: 0.75 with one
+// 128-column CTA per SM, 0.93 with two, 1.2 with three (a service warp counts half).  More items than resident
+// CTAs run in rounds.  FP64 rows share the SM's FP64 pipe, so the fullest SM's rows
+// add up (halo rows only pass through psi: 2 for the four), and one CTA alone leaves
+// the pipe idle for an eighth of the time.
+// Heights below 8 (the least before) pay on lattices that do not fill the chip: us
+// per step at 8 rows / at the model's choice: 512^2 FP32 12.3 / 10.8 (5 rows), 48
+// cells of 64^2 12.3 / 10.6 (6), 512^2 FP16 13.5 / 11.9 (5), FP64 177 / 161 (14).
+// A narrower last strip counts as a strip: leaving it out gave 1000 x 1000 FP32
+// 16-row segments in two rounds, 38.4 us, where 18 rows take one, 30.0 us.
+static int pick_segment_rows(const Geom& g, int nrows, int tile_x, int elem, int sms, int occ)
 {
     const long long strips = (g.nx + tile_x - 1) / tile_x;
     int best = 32;
     double best_cost = 1e300;
-    for (int ty = 8; ty <= 256 && ty <= nrows; ++ty) {
+    for (int ty = 2; ty <= 256 && ty <= nrows; ++ty) {
         const long long items = strips * g.n_cells * ((nrows + ty - 1) / ty);
-        const long long rounds = (items + slots - 1) / slots;
-        const int rows = std::min(ty, nrows);
-        const double cost = (double)rounds * (rows + 6);
+        const long long per_sm = (items + sms - 1) / sms;  // items of the fullest SM
+        double cost;
+        if (elem == 8) {
+            cost = (double)per_sm * (ty + 2) * (per_sm == 1 ? 1.13 : 1.0);
+        } else {
+            const long long rounds = (items + (long long)sms * occ - 1) / ((long long)sms * occ);
+            const double warps = (double)std::min<long long>(per_sm, occ) * (tile_x / 32 + 0.5);
+            cost = (double)rounds * (ty + 5.5) * (0.6 + 0.04 * warps);
+        }
         if (cost < best_cost - 1e-9) {
             best_cost = cost;
             best = ty;
@@ -216,8 +229,8 @@ TiledPlan* tiled_create(const Geom& g, const RowMap& rm, int prec, int elem, int
         occ[fam][smp] = o;
     }
     // segment height for the plain kernel of the family that will run most
-    const long long slots = (long long)sms * occ[any ? FAM_ANY : full_ok ? FAM_FULL : FAM_GEN][0];
-    if (p->ty <= 0) p->ty = pick_segment_rows(g, rm.nown, tile_x, slots);
+    if (p->ty <= 0)
+        p->ty = pick_segment_rows(g, rm.nown, tile_x, elem, sms, occ[any ? FAM_ANY : full_ok ? FAM_FULL : FAM_GEN][0]);
     p->n_seg = (rm.nown + p->ty - 1) / p->ty;
     const long long items = (long long)p->n_strips * p->n_seg * g.n_cells;
     for (int fam = 0; fam < N_FAM; ++fam)

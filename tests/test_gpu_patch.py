@@ -46,7 +46,7 @@ def run(cells, prec, kernel, pieces, sampling):
 @pytest.mark.parametrize("nx,ny,bc,n,model,pieces", [
     (64, 64, 1, 1, "paper", (1, 2, 7)), (32, 5, 0, 2, "forced", (9,)), (40, 9, 1, 3, "two_tau", (3, 6)),
     (72, 17, 0, 1, "mrt", (10,)), (320, 33, 1, 1, "paper", (8,)), (64, 16, 1, 2, "paper", (513, 2)),
-    (256, 511, 1, 1, "paper", (4,)), (64, 64, 1, 31, "two_tau", (5,))])
+    (256, 255, 1, 1, "paper", (4,)), (64, 64, 1, 15, "two_tau", (5,))])
 def test_equals_tiled_kernel_bitwise(prec, nx, ny, bc, n, model, pieces):
     cells = cells_of(nx, ny, bc, n, model)
     fa, oa, la, na = run(cells, prec, "auto", pieces, (2, 3))
