@@ -9,46 +9,20 @@
 
 namespace lbhb {
 
-// Two adjacent columns of one species per thread: vector (8-byte for FP32)
-// shared-memory accesses and two independent sites per thread.
+// Stores of two adjacent columns of one species (8 bytes for FP32).
 template <class T> struct Vec2;
 template <> struct Vec2<float> {
-    __device__ static void ld(const float* p, float& a, float& b)
-    {
-        const float2 v = *reinterpret_cast<const float2*>(p);
-        a = v.x;
-        b = v.y;
-    }
     __device__ static void st(float* p, float a, float b) { *reinterpret_cast<float2*>(p) = make_float2(a, b); }
 };
 template <> struct Vec2<double> {
-    __device__ static void ld(const double* p, double& a, double& b)
-    {
-        const double2 v = *reinterpret_cast<const double2*>(p);
-        a = v.x;
-        b = v.y;
-    }
     __device__ static void st(double* p, double a, double b) { *reinterpret_cast<double2*>(p) = make_double2(a, b); }
 };
 template <> struct Vec2<__half> {
-    __device__ static void ld(const __half* p, float& a, float& b)
-    {
-        const __half2 v = *reinterpret_cast<const __half2*>(p);
-        a = __low2float(v);
-        b = __high2float(v);
-    }
     // FP16 storage of shifted values: the caller subtracts the shift
     __device__ static void st(__half* p, float a, float b) { *reinterpret_cast<__half2*>(p) = __floats2half2_rn(a, b); }
 };
-// stochastically rounded FP16: loads as for __half (the caller unscales),
-// stores with the thread's dither stream
+// stochastically rounded FP16: stores with the thread's dither stream
 template <> struct Vec2<half_sr> {
-    __device__ static void ld(const half_sr* p, float& a, float& b)
-    {
-        const __half2 v = *reinterpret_cast<const __half2*>(p);
-        a = __low2float(v);
-        b = __high2float(v);
-    }
     __device__ static void st(half_sr* p, float a, float b, Dither& d)
     {
         const __half lo = half_sr_round(a, d), hi = half_sr_round(b, d);

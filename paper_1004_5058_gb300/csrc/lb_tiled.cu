@@ -36,6 +36,7 @@ struct TiledPlan {
     int elem, bc, tx, ty, depth;
     int n_strips, n_seg;
     bool any;        // any width: the FAM_ANY kernels
+    bool big;        // full_big
     int grid[N_FAM][2];  // persistent CTAs: [kernel family FAM_*][plain 0 / sampled 1]
     size_t smem;
     CUtensorMap tm_main[2], tm_halo[2];
@@ -140,13 +141,24 @@ static const void* pick_any(int prec, int tx, bool sample, int fam)
     }
 }
 
+// Whether FAM_FULL launches run as FAM_FULL_BIG: FP32 in 128-column tiles whose two
+// buffers are more than twice the L2 (129 MB), so that a step streams from memory and
+// rows that finish sooner only spread the CTAs' accesses.  us per step, FAM_FULL /
+// FAM_FULL_BIG: 1024^2 (151 MB) 28.4 / 28.8, 16 x 512^2 (302 MB) 101.4 / 100.9,
+// 8 x 1024^2 (604 MB) 202.0 / 199.9; 1024 x 64^2 (604 MB, 64 columns) 118.8 / 122.3.
+static bool full_big(const Geom& g, int prec, int tile_x)
+{
+    return prec == LB_FP32 && tile_x == 128 && 2 * 18 * g.plane * g.n_cells * 4 > (256LL << 20);
+}
+
 // The family a launch runs: the full-width one when the strips are whole and
 // every cell has one relaxation time and BGK, else the general or MRT one.
 static int launch_family(const TiledPlan* p)
 {
     if (p->any) return p->collision == TILED_MRT ? FAM_ANY_MRT : FAM_ANY;
     if (p->collision == TILED_MRT) return FAM_MRT;
-    return p->g.nx % p->tx == 0 && p->collision == TILED_BGK_ONE_TIME ? FAM_FULL : FAM_GEN;
+    if (p->g.nx % p->tx != 0 || p->collision != TILED_BGK_ONE_TIME) return FAM_GEN;
+    return p->big ? FAM_FULL_BIG : FAM_FULL;
 }
 
 static bool encode(CUtensorMap* m, void* base, const Geom& g, int elem, int box_x)
@@ -182,6 +194,7 @@ TiledPlan* tiled_create(const Geom& g, const RowMap& rm, int prec, int elem, int
     p->any = any;
     p->tx = tile_x;
     p->ty = tile_y;
+    p->big = full_big(g, prec, tile_x);
     p->depth = depth_for(tile_x, elem);
     p->n_strips = (g.nx + tile_x - 1) / tile_x;
     p->smem = smem_bytes(tile_x, elem, p->depth);
@@ -204,10 +217,11 @@ TiledPlan* tiled_create(const Geom& g, const RowMap& rm, int prec, int elem, int
     // share the work items (the segment height) but each runs as many persistent
     // CTAs as fit (the sampled variant holds more registers)
     const bool full_ok = g.nx % tile_x == 0;
+    const int full = p->big ? FAM_FULL_BIG : FAM_FULL, no_full = p->big ? FAM_FULL : FAM_FULL_BIG;
     int occ[N_FAM][2] = {};
     for (int s = 0; s < 2 * N_FAM; ++s) {
         const int fam = s >> 1, smp = s & 1;
-        if (any != (fam >= FAM_ANY) || (fam == FAM_FULL && !full_ok)) continue;
+        if (any != (fam >= FAM_ANY) || (fam == full && !full_ok) || fam == no_full) continue;
         const void* k = pick_any(prec, tile_x, smp != 0, fam);
         // the whole unified L1/shared array as shared memory: the CTAs' rings
         // are what sets how many fit on an SM
@@ -230,7 +244,7 @@ TiledPlan* tiled_create(const Geom& g, const RowMap& rm, int prec, int elem, int
     }
     // segment height for the plain kernel of the family that will run most
     if (p->ty <= 0)
-        p->ty = pick_segment_rows(g, rm.nown, tile_x, elem, sms, occ[any ? FAM_ANY : full_ok ? FAM_FULL : FAM_GEN][0]);
+        p->ty = pick_segment_rows(g, rm.nown, tile_x, elem, sms, occ[any ? FAM_ANY : full_ok ? full : FAM_GEN][0]);
     p->n_seg = (rm.nown + p->ty - 1) / p->ty;
     const long long items = (long long)p->n_strips * p->n_seg * g.n_cells;
     for (int fam = 0; fam < N_FAM; ++fam)

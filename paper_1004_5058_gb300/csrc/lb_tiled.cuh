@@ -97,6 +97,8 @@ __device__ __noinline__ void profile_row_sums(const C* ub, int lane, double* __r
 // Kernel families (FAM):
 //   FAM_FULL  every strip is TX columns wide (nx a multiple of TX) and every cell
 //             has one relaxation time (BGK);
+//   FAM_FULL_BIG  the same, for lattices far larger than the L2 (full_big): ring rows
+//             are computed per row instead of kept, stores without the streaming hint;
 //   FAM_GEN   the last strip may be narrower (its extra columns masked) and the
 //             species may relax with times of their own (BGK);
 //   FAM_MRT   as FAM_GEN, with the multiple-relaxation-time collision;
@@ -106,7 +108,7 @@ __device__ __noinline__ void profile_row_sums(const C* ub, int lane, double* __r
 //             last pair of an odd width updates its first site only.  1021 x 509
 //             FP32 18.8 us per step where the generic pair takes 39.5 (its two
 //             passes move 232 bytes per site and its loads wait one by one).
-constexpr int FAM_FULL = 0, FAM_GEN = 1, FAM_MRT = 2, FAM_ANY = 3, FAM_ANY_MRT = 4, N_FAM = 5;
+constexpr int FAM_FULL = 0, FAM_FULL_BIG = 1, FAM_GEN = 2, FAM_MRT = 3, FAM_ANY = 4, FAM_ANY_MRT = 5, N_FAM = 6;
 template <class T, int TX, bool SAMPLE, int FAM>
 __global__ void __launch_bounds__(tiled_threads(TX),
                                   SAMPLE ? (tiled_min_ctas(TX, (int)sizeof(T)) < 3 ? tiled_min_ctas(TX, (int)sizeof(T)) : 3)
@@ -124,7 +126,11 @@ __global__ void __launch_bounds__(tiled_threads(TX),
 {
     using C = typename Store<T>::C;
     using V = P2<C>;  // a lane pair: one species at the thread's two sites
-    constexpr bool FULL = FAM == FAM_FULL, MRT = FAM == FAM_MRT || FAM == FAM_ANY_MRT, ANY = FAM >= FAM_ANY;
+    constexpr bool FULL = FAM == FAM_FULL || FAM == FAM_FULL_BIG, MRT = FAM == FAM_MRT || FAM == FAM_ANY_MRT, ANY = FAM >= FAM_ANY;
+    // Ring rows kept in registers and streaming stores of the whole pairs: FP32, 8 x
+    // 1024^2 MRT 216.4 -> 209.6 us, 48 x 64^2 10.5 -> 10.3, 1021 x 509 18.4 -> 18.0;
+    // FP16, at its register limit, loses 1.5 %, and so does the memory-bound FAM_FULL_BIG
+    constexpr bool KEEP = std::is_same<T, float>::value && FAM != FAM_FULL_BIG;
     // stored populations are scale * g (scale 1 except for the dithered FP16 storage)
     constexpr C scale = C(Store<T>::scale), inv_scale = C(1) / scale;
     constexpr int E = (int)sizeof(T);
@@ -140,9 +146,10 @@ __global__ void __launch_bounds__(tiled_threads(TX),
 
     extern __shared__ __align__(128) unsigned char smem[];
     unsigned char* fring = smem;
-    C* psi_ring = reinterpret_cast<C*>(smem + D * SLOT);  // [species][RING][W] (stride SS per species)
-    C* rho_ring = psi_ring + 2 * SS;
-    uint64_t* bars = reinterpret_cast<uint64_t*>(rho_ring + 2 * SS);
+    // rings [RING][W], SS apart: psi of A, rho of B, psi of B, rho of A, so that a
+    // lane's psi and its partner's rho lie at one distance from each other
+    unsigned char* const rings = smem + D * SLOT;
+    uint64_t* bars = reinterpret_cast<uint64_t*>(rings + 4 * SS * (int)sizeof(C));
     // sampled steps: u_x of each site of the last two rows, summed by the service warp
     C* ubuf = reinterpret_cast<C*>(bars + D);
 
@@ -292,18 +299,23 @@ __global__ void __launch_bounds__(tiled_threads(TX),
         bad = false;
 
         if (issuer) issue_upto(nrow + D);  // rows of earlier items are all done
-        auto wait_row = [&](int k) -> bool {
-            const uint32_t n = nrow + (uint32_t)k;
-            return mbar_wait_bounded(&bars[n % D], (n / D) & 1u);
-        };
-        // rho_s, psi_s of logical row k into ring row `ring_row` (own species,
-        // own two columns; the service warp takes the halo columns)
-        auto psi_stage_slot = [&](int slot, int ring_row) {
-            const unsigned char* base = fring + slot * SLOT;
-            const int ring = sp * SS + ring_row * W;
+        // Byte offsets of this thread, advanced by one row per iteration instead of
+        // computed from row numbers: its place in a ring row (two columns left of the
+        // lane's first; the service warp: of its halo column) and in a row slot
+        constexpr int RW = W * (int)sizeof(C);                           // a ring row
+        constexpr int PARTNER = SS * (int)sizeof(C);                     // from psi to the partner's rho
+        const int own = (sp ? -SS : 3 * SS) * (int)sizeof(C);            // from psi to the lane's own rho
+        const int hpos = (lane & 3) < 2 ? lane & 3 : wv + (lane & 3);    // service warp
+        const int ring0 = (sp * 2 * SS + (svc ? hpos - 2 : c0)) * (int)sizeof(C), ring_end = ring0 + RING * RW;
+        const int slot0 = svc ? 0 : (sp * 9 * TX + c0) * E;
+        // rho_s, psi_s of the row in the slot at `slot` into the ring row at `ring` (own
+        // species, own two columns; the service warp takes the halo columns)
+        auto psi_stage = [&](int slot, int ring) {
+            C* const to = reinterpret_cast<C*>(rings + ring) + 2;
+            C* const to_rho = reinterpret_cast<C*>(rings + ring + own) + 2;
             if (!svc) {
                 if (!act) return;  // its ring positions belong to the halo or to nobody
-                const T* src = reinterpret_cast<const T*>(base) + sp * 9 * TX + c0;
+                const T* src = reinterpret_cast<const T*>(fring + slot);
                 V r = Pair<T>::ld(src);
 #pragma unroll
                 for (int i = 1; i < 9; ++i) r = r + Pair<T>::ld(src + i * TX);
@@ -315,15 +327,16 @@ __global__ void __launch_bounds__(tiled_threads(TX),
                 }
                 const V ps = lane_psi(r, rho0_2, inv_rho0_2);
                 if (ANY && !act_b) {  // the next position is a halo column
-                    psi_ring[ring + c0 + 2] = ps.a();
-                    rho_ring[ring + c0 + 2] = r.a();
+                    *to = ps.a();
+                    *to_rho = r.a();
                 } else {
-                    Pair<C>::st(psi_ring + ring + c0 + 2, ps);
-                    Pair<C>::st(rho_ring + ring + c0 + 2, r);
+                    Pair<C>::st(to, ps);
+                    Pair<C>::st(to_rho, r);
                 }
             } else if (lane < 8) {
                 // halo column h: 0,1 -> columns -2,-1 (left box); 2,3 -> TX, TX+1 (right box)
                 const int h = lane & 3;
+                const unsigned char* const base = fring + slot;
                 const T* src = reinterpret_cast<const T*>(base + (h < 2 ? MAIN_AL : MAIN_AL + HALO_AL)) + sp * 9 * H +
                                (h < 2 ? H - 2 + h : h - 2);
                 C acc = C(0);
@@ -336,16 +349,28 @@ __global__ void __launch_bounds__(tiled_threads(TX),
                         acc += to_c(src[i * H]);
                 }
                 if (Store<T>::shifted) acc = acc * inv_scale + rho_bar;
-                const int pos = h < 2 ? h : wv + h;
-                psi_ring[ring + pos] = psi_of(acc, p.rho0, p.inv_rho0);
-                rho_ring[ring + pos] = acc;
+                *to = psi_of(acc, p.rho0, p.inv_rho0);
+                *to_rho = acc;
             }
         };
 
         bool ok = true;
+        // slot, and the phase of its barrier, of the row that is staged next (global row nrow + k)
+        int sb = (int)(nrow % (uint32_t)D);
+        uint32_t ph = (nrow / (uint32_t)D) & 1u;
+        auto next_slot = [&]() {
+            if (++sb == D) {
+                sb = 0;
+                ph ^= 1u;
+            }
+        };
+        // Ring rows of logical rows j .. j + 4, read by the collision of row j + 2: all
+        // five kept and rotated where registers are free (KEEP), else four of them from the first
+        int rr[5] = {ring0, ring0 + RW, ring0 + 2 * RW, ring0 + 3 * RW, ring0 + 4 * RW};
         for (int k = 0; k < 4; ++k) {
-            ok = wait_row(k) && ok;
-            psi_stage_slot((int)((nrow + (uint32_t)k) % (uint32_t)D), k);
+            ok = mbar_wait_bounded(&bars[sb], ph) && ok;
+            psi_stage(slot0 + sb * SLOT, ring0 + k * RW);
+            next_slot();
         }
         if constexpr (D < 5) {
             // a four-slot ring holds rows 0..3 only: rows 4 and 5 go into the slots of
@@ -354,23 +379,18 @@ __global__ void __launch_bounds__(tiled_threads(TX),
             __syncthreads();
             if (issuer) issue_upto(nrow + 2u + (uint32_t)D);
         }
-        int r0 = 0;  // ring row of logical row j (rows j .. j+4 are read by the collision of row j+2)
-        // slot and mbarrier phase of logical row j + 4 (global row nrow + j + 4),
-        // advanced by one row per iteration instead of recomputed
-        int s4 = (int)((nrow + 4u) % (uint32_t)D);
-        uint32_t ph4 = ((nrow + 4u) / (uint32_t)D) & 1u;
         for (int j = 0; j < rows; ++j) {
-            int rr[5];
+            int ring_row[5];
 #pragma unroll
-            for (int d = 0; d < 5; ++d) rr[d] = r0 + d >= RING ? r0 + d - RING : r0 + d;
-            const int s2 = s4 >= 2 ? s4 - 2 : s4 + D - 2;  // slot of row j + 2
-            ok = mbar_wait_bounded(&bars[s4], ph4) && ok;
-            psi_stage_slot(s4, rr[4]);
-            if (++s4 == D) {
-                s4 = 0;
-                ph4 ^= 1u;
-            }
-            r0 = rr[1];
+            for (int d = 0; d < 5; ++d)
+                ring_row[d] = KEEP ? rr[d] : rr[0] + d * RW >= ring_end ? rr[0] + (d - RING) * RW : rr[0] + d * RW;
+            const int s2 = slot0 + (sb >= 2 ? sb - 2 : sb + D - 2) * SLOT;  // slot of row j + 2
+            ok = mbar_wait_bounded(&bars[sb], ph) && ok;
+            psi_stage(slot0 + sb * SLOT, ring_row[4]);
+            next_slot();
+#pragma unroll
+            for (int d = 0; d < 4; ++d) rr[d] = ring_row[d + 1];
+            rr[4] = ring_row[4] + RW == ring_end ? ring0 : ring_row[4] + RW;
             // barrier: psi/rho of row j+4 visible, collision of row j+1 finished
             // everywhere; it also tells every thread whether any wait ran out
             if (__syncthreads_or(ok ? 0 : 1)) {
@@ -387,7 +407,7 @@ __global__ void __launch_bounds__(tiled_threads(TX),
             }
             // ---- collide logical row k = j + 2 (lattice row y), sites x and x+1
             const int y = y0 + j, gy = y - rm.ylo + rm.y0g;  // buffer row, row of the global cell
-            const T* fm = reinterpret_cast<const T*>(fring + s2 * SLOT) + sp * 9 * TX + c0;
+            const T* fm = reinterpret_cast<const T*>(fring + s2);
             // populations as stored: f for FP32/FP64, the shifted g for FP16; a
             // lane pair per direction (sites x, x+1)
             V f[9];
@@ -395,18 +415,17 @@ __global__ void __launch_bounds__(tiled_threads(TX),
             for (int i = 0; i < 9; ++i) f[i] = Pair<T>::ld(fm + i * TX);
             // psi window rows k-2..k+2 and rho_s' window rows k-1..k+1, columns
             // c0-2..c0+3 as three pairs; window column 2 + o is site o
-            const C* ps = psi_ring + sp * SS + c0;  // ring column c0 + 2 + dx  <->  column c0 + dx
-            const C* ro = rho_ring + (1 - sp) * SS + c0;
             V v[5][3], e[3][3];
 #pragma unroll
-            for (int d = 0; d < 5; ++d)
+            for (int d = 0; d < 5; ++d) {
+                const C* const ps = reinterpret_cast<const C*>(rings + ring_row[d]);
 #pragma unroll
-                for (int m = 0; m < 3; ++m) v[d][m] = Pair<C>::ld(ps + rr[d] * W + 2 * m);
+                for (int m = 0; m < 3; ++m) v[d][m] = Pair<C>::ld(ps + 2 * m);
+                if (d == 0 || d == 4) continue;
 #pragma unroll
-            for (int d = 0; d < 3; ++d)
-#pragma unroll
-                for (int m = 0; m < 3; ++m) e[d][m] = Pair<C>::ld(ro + rr[d + 1] * W + 2 * m);
-            const V rho_s = Pair<C>::ld(rho_ring + sp * SS + rr[2] * W + c0 + 2);
+                for (int m = 0; m < 3; ++m) e[d - 1][m] = Pair<C>::ld(ps + PARTNER / (int)sizeof(C) + 2 * m);
+            }
+            const V rho_s = Pair<C>::ld(reinterpret_cast<const C*>(rings + ring_row[2] + own) + 2);
             const V rho_p = e[1][1];  // the partner species' densities at the same two sites
             // pair differences d_q = psi(r + c_q) - psi(r - c_q) of both sites
             V dps[12], dro[4];
@@ -485,7 +504,10 @@ __global__ void __launch_bounds__(tiled_threads(TX),
                         const int cy = q_cy(i), cx = q_cx(i);
                         T* const q = dst_x + (i * pl + row3[cy + 1]);
                         if (cx == 0) {
-                            st_pair<T, C>(q, fs[i].a(), fs[i].b(), dz);
+                            if constexpr (KEEP)  // whole sectors: first out of the L2
+                                __stcs(reinterpret_cast<float2*>(q), make_float2(fs[i].a(), fs[i].b()));
+                            else
+                                st_pair<T, C>(q, fs[i].a(), fs[i].b(), dz);
                         } else {
                             st_one<T, C>(q + cx, fs[i].a(), dz);
                             st_one<T, C>(q + cx + 1, fs[i].b(), dz);
@@ -597,6 +619,8 @@ static const void* kernel_ptr(bool sample, int fam)
         if (fam == FAM_ANY) return kernel_ptr<T, TX, FAM_ANY>(sample);
         if (fam == FAM_ANY_MRT) return kernel_ptr<T, TX, FAM_ANY_MRT>(sample);
     }
+    if constexpr (std::is_same<T, float>::value && TX == 128)  // full_big
+        if (fam == FAM_FULL_BIG) return kernel_ptr<T, TX, FAM_FULL_BIG>(sample);
     return fam == FAM_FULL ? kernel_ptr<T, TX, FAM_FULL>(sample)
          : fam == FAM_GEN  ? kernel_ptr<T, TX, FAM_GEN>(sample)
                            : kernel_ptr<T, TX, FAM_MRT>(sample);
