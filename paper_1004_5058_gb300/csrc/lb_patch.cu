@@ -310,7 +310,7 @@ __global__ void __launch_bounds__(PATCH_THREADS) patch_steps_kernel(const __grid
             const C fx_body = body_force_x<C>(pg, y);
             const V rho_t = rho_s + rho_p;
             V ax = V(fx_body) * inv_rho;
-            if (!one_time && fx_body != C(0)) ax = V(fx_body) * lane_rcp(rho_t);
+            if (!one_time && !is_zero(fx_body)) ax = V(fx_body) * lane_rcp(rho_t);
             bad |= (act_a && !density_ok(first(rho_t))) ||
                    (act_b && !density_ok(second(rho_t)));
             V fs[9], Fx;

@@ -452,7 +452,7 @@ __global__ void __launch_bounds__(tiled_threads(TX),
             const V inv_rho = lane_rcp(rho_w);
             const V ux = jwx * inv_rho, uy = jwy * inv_rho;
             const C fx_body = body_force_x<C>(p, gy);
-            const bool body_raw = !one_time && fx_body != C(0);  // the force needs the raw 1/rho
+            const bool body_raw = !one_time && !is_zero(fx_body);  // the force needs the raw 1/rho
             const V rho_t = FULL ? rho_w : rho_s + rho_p;        // total density of each site
             V ax = V(fx_body) * inv_rho;
             if (body_raw) ax = V(fx_body) * lane_rcp(rho_t);
