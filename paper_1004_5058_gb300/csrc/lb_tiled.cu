@@ -144,8 +144,11 @@ static const void* pick_any(int prec, int tx, bool sample, int fam)
 // Whether FAM_FULL launches run as FAM_FULL_BIG: FP32 in 128-column tiles whose two
 // buffers are more than twice the L2 (129 MB), so that a step streams from memory and
 // rows that finish sooner only spread the CTAs' accesses.  us per step, FAM_FULL /
-// FAM_FULL_BIG: 1024^2 (151 MB) 28.4 / 28.8, 16 x 512^2 (302 MB) 101.4 / 100.9,
-// 8 x 1024^2 (604 MB) 202.0 / 199.9; 1024 x 64^2 (604 MB, 64 columns) 118.8 / 122.3.
+// FAM_FULL_BIG: 1024^2 (151 MB) 28.4 / 28.8, 16 x 512^2 (604 MB) 101.4 / 100.9,
+// 8 x 1024^2 (1.2 GB) 202.0 / 199.9; 1024 x 64^2 (604 MB, 64 columns) 118.8 / 122.3.
+// Their row copies also fetch 256 bytes into the L2 at a time, where 128 serve the
+// others: 128 / 256 bytes, 8 x 1024^2 202.0 / 200.9, 16 x 512^2 101.7 / 101.4, two
+// relaxation times 200.9 / 199.8, 4096^2 419 / 421; 512^2, which the L2 holds, 10.67 / 10.78.
 static bool full_big(const Geom& g, int prec, int tile_x)
 {
     return prec == LB_FP32 && tile_x == 128 && 2 * 18 * g.plane * g.n_cells * 4 > (256LL << 20);
@@ -161,7 +164,7 @@ static int launch_family(const TiledPlan* p)
     return p->big ? FAM_FULL_BIG : FAM_FULL;
 }
 
-static bool encode(CUtensorMap* m, void* base, const Geom& g, int elem, int box_x)
+static bool encode(CUtensorMap* m, void* base, const Geom& g, int elem, int box_x, bool big)
 {
     auto fn = encode_fn();
     if (!fn) return false;
@@ -174,7 +177,7 @@ static bool encode(CUtensorMap* m, void* base, const Geom& g, int elem, int box_
     cuuint32_t box[4] = {(cuuint32_t)box_x, 1, 18, 1};
     cuuint32_t es[4] = {1, 1, 1, 1};
     CUresult r = fn(m, dt, 4, base, dims, strides, box, es, CU_TENSOR_MAP_INTERLEAVE_NONE,
-                    CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
+                    CU_TENSOR_MAP_SWIZZLE_NONE, big ? CU_TENSOR_MAP_L2_PROMOTION_L2_256B : CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
                     CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
     return r == CUDA_SUCCESS;
 }
@@ -202,7 +205,8 @@ TiledPlan* tiled_create(const Geom& g, const RowMap& rm, int prec, int elem, int
     p->f[1] = f1;
     const int halo = 16 / elem;
     for (int b = 0; b < 2; ++b)
-        if (!encode(&p->tm_main[b], b ? f1 : f0, g, elem, tile_x) || !encode(&p->tm_halo[b], b ? f1 : f0, g, elem, halo)) {
+        if (!encode(&p->tm_main[b], b ? f1 : f0, g, elem, tile_x, p->big) ||
+            !encode(&p->tm_halo[b], b ? f1 : f0, g, elem, halo, p->big)) {
             if (err_msg) *err_msg = "cuTensorMapEncodeTiled failed";
             delete p;
             return nullptr;

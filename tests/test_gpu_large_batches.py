@@ -23,7 +23,7 @@ def run(cells, fields):
         return lat.get_populations(), lat.profile()[0]
 
 
-# 2 x 2 x 18 x 4 bytes per site: 256 MB are 1.864e6 sites; the sizes lie just above, with whole strips
+# both buffers hold 2 x 18 x 4 bytes per site: 256 MB are 1.864e6 sites; the sizes lie just above, in whole strips
 @pytest.mark.parametrize("bc,f0", [(1, 0.0), (0, 1e-5)])
 @pytest.mark.parametrize("nx,ny", [(1024, 911), (1152, 811), (128, 7283)])
 def test_cells_of_a_large_batch_equal_single_cells(nx, ny, bc, f0):
