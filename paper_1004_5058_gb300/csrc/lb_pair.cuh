@@ -1,5 +1,5 @@
 // Device helpers of the kernels whose threads hold one species at two adjacent
-// sites (lb_tiled.cu, lb_patch.cu): stores of a pair in each storage format and
+// sites (lb_tiled.cuh, lb_patch.cu): stores of a pair in each storage format and
 // the differences of Eq. (FFF) over a window of psi/rho pairs.
 #pragma once
 

@@ -1,6 +1,6 @@
 // Patch kernel: many time steps of a small lattice in one launch.
 //
-// The tiled kernel (lb_tiled.cu) walks rows: a segment costs its rows plus six
+// The tiled kernel (lb_tiled.cuh) walks rows: a segment costs its rows plus six
 // one after another, however few there are, and every step is a launch.  A
 // lattice of 64^2 sites then keeps 8 SMs busy for 12 rows.  Here a thread block
 // takes a patch of BX x BY sites and updates all of it at once, so the whole
