@@ -292,14 +292,18 @@ static void drop_auto(lb_handle* h)
 //         101 x 83 (generic pair) 24 / 12, 201 x 163 (generic pair) 24.4 / 26.5.
 // The patch kernel's time grows with the sites each SM holds; they meet near 2^16
 // sites in FP32 and FP16, 2^17 in FP64, and 2^15 with the FP64 generic pair.
-// Larger FP32 and FP16 lattices whose width lb_set_kernel refuses to the tiled
-// kernel run its any-width form instead of the generic pair (us per step, generic
-// / any width: 1021 x 509 FP32 39.5 / 18.8, FP16 44.7 / 22.1; 1021 x 1509 123 / 50;
-// 401 x 399 15.8 / 14.4; 16 cells of 101 x 260 41.5 / 22.0).  FP64 stays with the
-// pair: its pipe bounds both (1021 x 509 293 us).
+// Larger FP32 lattices whose width lb_set_kernel refuses to the tiled kernel run
+// its any-width form instead of the generic pair (us per step, generic / any width:
+// 1021 x 509 39.5 / 18.8; 1021 x 1509 123 / 50; 401 x 399 15.8 / 14.4; 16 cells of
+// 101 x 260 41.5 / 22.0).  FP64 stays with the pair: its pipe bounds both (1021 x
+// 509 293 us).
+// FP16 storage of such widths stays with the pair at every size: both kernels above
+// group their FP32 sums otherwise, the last FP32 bit decides FP16 roundings, and
+// dithered storage draws its bits per pair of sites there, so the outputs of a run
+// would be others (by 4e-4 after 60 steps) than the pair's.
 static void select_beyond_family(lb_handle* h)
 {
-    if (h->slab) return;
+    if (h->slab || (h->elem == 2 && h->kernel == LB_KERNEL_GENERIC)) return;
     const long long most = h->prec != LB_FP64 ? 1LL << 16 : h->kernel == LB_KERNEL_GENERIC ? 1LL << 15 : 1LL << 17;
     if ((long long)h->n_cells * h->nx * h->ny < most) {
         h->patch = patch_create(h->g, (int)h->prec, h->bc);

@@ -16,7 +16,7 @@ int generic_partials_nbx(const Geom& g);
 struct TiledPlan;  // opaque per-handle state of the tiled kernel
 bool tiled_supported(const Geom& g, int elem_bytes, int tile_x, int tile_y);
 // Any width of at least tile_x (64 or 128) columns, odd ones too (whole cells, FP32
-// and FP16 storage): LB_KERNEL_AUTO runs it where tiled_supported says no.
+// storage): LB_KERNEL_AUTO runs it where tiled_supported says no.
 bool tiled_any_supported(const Geom& g, int elem_bytes, int tile_x);
 int tiled_partials_nbx(const Geom& g, int tile_x);
 // Creates the plan (tensor maps for both ping-pong buffers).  Returns nullptr

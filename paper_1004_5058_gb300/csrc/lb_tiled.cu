@@ -125,7 +125,7 @@ bool tiled_supported(const Geom& g, int elem, int tile_x, int tile_y)
 
 bool tiled_any_supported(const Geom& g, int elem, int tile_x)
 {
-    return elem < 8 && (tile_x == 64 || tile_x == 128) && g.nx >= tile_x && g.ny >= 5 && 18 * g.plane < (1LL << 31) &&
+    return elem == 4 && (tile_x == 64 || tile_x == 128) && g.nx >= tile_x && g.ny >= 5 && 18 * g.plane < (1LL << 31) &&
            encode_fn() != nullptr;
 }
 

@@ -102,10 +102,10 @@ __device__ __noinline__ void profile_row_sums(const C* ub, int lane, double* __r
 //   FAM_GEN   the last strip may be narrower (its extra columns masked) and the
 //             species may relax with times of their own (BGK);
 //   FAM_MRT   as FAM_GEN, with the multiple-relaxation-time collision;
-//   FAM_ANY, FAM_ANY_MRT  as these for any width, odd ones too.  The halo columns of
-//             such a row have no aligned place for a TMA box: the service warp
-//             copies them word by word (cp.async, on the row's mbarrier), and the
-//             last pair of an odd width updates its first site only.  1021 x 509
+//   FAM_ANY, FAM_ANY_MRT  as these for any width, odd ones too, in FP32 storage.  The
+//             halo columns of such a row have no aligned place for a TMA box: the
+//             service warp copies them word by word (cp.async, on the row's mbarrier),
+//             and the last pair of an odd width updates its first site only.  1021 x 509
 //             FP32 18.8 us per step where the generic pair takes 39.5 (its two
 //             passes move 232 bytes per site and its loads wait one by one).
 constexpr int FAM_FULL = 0, FAM_FULL_BIG = 1, FAM_GEN = 2, FAM_MRT = 3, FAM_ANY = 4, FAM_ANY_MRT = 5, N_FAM = 6;
@@ -142,7 +142,7 @@ __global__ void __launch_bounds__(tiled_threads(TX),
     constexpr int HALO_AL = al128(18 * H * E);
     constexpr int SLOT = MAIN_AL + 2 * HALO_AL;
     constexpr uint32_t TX_BYTES = 18 * TX * E + (ANY ? 0 : 2 * 18 * H * E);
-    constexpr int PER_WORD = 4 / E > 0 ? 4 / E : 1;  // ANY: columns in a 4-byte halo word
+    static_assert(!ANY || std::is_same<T, float>::value, "a halo column of the any-width form is one 4-byte word");
 
     extern __shared__ __align__(128) unsigned char smem[];
     unsigned char* fring = smem;
@@ -222,8 +222,7 @@ __global__ void __launch_bounds__(tiled_threads(TX),
                 }
                 if constexpr (ANY) {
                     // word (population q, halo column h) at 4 q + h, h = lane & 3
-                    const T* const row = fin + (long long)icell * g.cellstride + (long long)yp * g.pitch +
-                                         (ihc & ~(PER_WORD - 1));
+                    const T* const row = fin + (long long)icell * g.cellstride + (long long)yp * g.pitch + ihc;
                     for (int e = lane; e < 72; e += 32)
                         cp_async4(dst + MAIN_AL + 4 * e, row + (long long)(e >> 2) * g.plane);
                     cp_async_arrive(&bars[slot]);
@@ -281,7 +280,6 @@ __global__ void __launch_bounds__(tiled_threads(TX),
         const int wv = FULL ? TX : min(TX, g.nx - x0);
         const bool act = FULL || c0 < wv;                 // the pair's first column
         const bool act_b = FULL || c0 + (ANY ? 1 : 0) < wv;  // its second (the same unless the width is odd)
-        const int hc = ANY && svc ? halo_column(x0) : 0;
         // destination columns of the two sites x, x+1 shifted by -1/0/+1 (periodic)
         const int x = x0 + c0;
         const int col_m = x == 0 ? g.nx - 1 : x - 1, col_p2 = x + 2 == g.nx ? 0 : x + 2;
@@ -343,8 +341,7 @@ __global__ void __launch_bounds__(tiled_threads(TX),
 #pragma unroll
                 for (int i = 0; i < 9; ++i) {
                     if constexpr (ANY)
-                        acc += to_c(reinterpret_cast<const T*>(base + MAIN_AL)[((sp * 9 + i) * 4 + h) * PER_WORD +
-                                                                                (hc & (PER_WORD - 1))]);
+                        acc += to_c(reinterpret_cast<const T*>(base + MAIN_AL)[(sp * 9 + i) * 4 + h]);
                     else
                         acc += to_c(src[i * H]);
                 }
@@ -615,7 +612,7 @@ static const void* kernel_ptr(bool sample)
 template <class T, int TX>
 static const void* kernel_ptr(bool sample, int fam)
 {
-    if constexpr (sizeof(T) < 8 && (TX == 64 || TX == 128)) {  // tiled_any_supported
+    if constexpr (std::is_same<T, float>::value && (TX == 64 || TX == 128)) {  // tiled_any_supported
         if (fam == FAM_ANY) return kernel_ptr<T, TX, FAM_ANY>(sample);
         if (fam == FAM_ANY_MRT) return kernel_ptr<T, TX, FAM_ANY_MRT>(sample);
     }
