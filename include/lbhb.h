@@ -149,7 +149,9 @@ lb_status lb_init_fields(lb_handle* h, const double* rho_a, const double* rho_b,
  * asynchronous (pageable memory is copied through a driver bounce buffer and
  * may make the call wait).  A second lb_stage_fields before
  * lb_init_fields_staged replaces the staged fields; lb_init_fields discards
- * them.  The first call allocates the staging buffer.
+ * them.  The first call allocates the staging buffer; lb_get_fields reads back
+ * through a buffer of its own (allocated when first needed) while fields are
+ * staged, and leaves them as they are.
  * lb_init_fields_staged waits on the host for the staged copy, then enqueues
  * f = f^eq of the staged fields on the handle's stream and returns without
  * synchronising; counters and time averages reset as in lb_init_fields.

@@ -56,6 +56,7 @@ struct lb_handle {
     double* red_part = nullptr;
     double* red_out = nullptr;
     double* staging = nullptr;         // [4][cell][ny][nx] float64: each host field is one copy
+    double* readback = nullptr;        // the same for lb_get_fields while staged fields fill `staging`
     cudaStream_t copy_stream = nullptr;  // lb_stage_fields' copies (created on first use)
     cudaEvent_t staged = nullptr;        // the last staged copy is complete
     cudaEvent_t staging_read = nullptr;  // the last equilibrium launch has read the staging buffer
@@ -130,6 +131,7 @@ static void release(lb_handle* h)
     cudaFree(h->red_part);
     cudaFree(h->red_out);
     cudaFree(h->staging);
+    cudaFree(h->readback);
     if (h->h_err) cudaFreeHost(h->h_err);
     if (h->batch_done) cudaEventDestroy(h->batch_done);
     if (h->copy_stream) {
@@ -1058,10 +1060,13 @@ lb_status lb_get_fields(lb_handle* h, double* rho_a, double* rho_b, double* ux, 
     if (!h->initialised) return fail(h, LB_ERR_STATE, "lb_get_fields: no state loaded");
     CK(h, cudaSetDevice(h->device));
     const size_t n = (size_t)h->nx * h->ny * h->n_cells;
-    if (!h->staging) CK(h, cudaMalloc(&h->staging, sizeof(double) * 4 * n));
+    // fields staged for the next run keep `staging`, which the copy stream may still be
+    // writing, until lb_init_fields_staged takes them
+    double*& buf = h->staged_pending ? h->readback : h->staging;
+    if (!buf) CK(h, cudaMalloc(&buf, sizeof(double) * 4 * n));
     CK(h, with_type(h, [&](auto* tp) {
         using T = std::remove_pointer_t<decltype(tp)>;
-        return launch_fields<T>((const T*)fview(h, h->cur), h->staging, h->g, h->d_cells, h->d_err, h->stream);
+        return launch_fields<T>((const T*)fview(h, h->cur), buf, h->g, h->d_cells, h->d_err, h->stream);
     }));
     h->launches += 1;
     // one contiguous copy per field: strided copies of 16 cells of 512^2 into pageable
@@ -1069,7 +1074,7 @@ lb_status lb_get_fields(lb_handle* h, double* rho_a, double* rho_b, double* ux, 
     double* dst[4] = {rho_a, rho_b, ux, uy};
     for (int a = 0; a < 4; ++a)
         if (dst[a])
-            CK(h, cudaMemcpyAsync(dst[a], h->staging + a * n, n * sizeof(double), cudaMemcpyDeviceToHost, h->stream));
+            CK(h, cudaMemcpyAsync(dst[a], buf + a * n, n * sizeof(double), cudaMemcpyDeviceToHost, h->stream));
     return sync_and_check(h);
 }
 
