@@ -57,7 +57,8 @@ lb_status mlp_create(const mlp_config* cfg, void* cuda_stream, mlp_handle** out)
 lb_status mlp_set_params(mlp_handle* h, const float* params, long long n);
 lb_status mlp_get_params(mlp_handle* h, float* params, long long n);
 
-/* Forward pass: x [B][5] raw inputs -> out [B][2] = (stress, logit).  Async. */
+/* Forward pass: x [B][5] raw inputs -> out [B][2] = (stress, logit); out may
+ * overlap x.  Async. */
 lb_status mlp_forward(mlp_handle* h, const float* x, int batch, float* out);
 
 /* Loss and its gradient with respect to every parameter, without updating:

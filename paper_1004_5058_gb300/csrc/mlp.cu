@@ -743,6 +743,7 @@ struct mlp_handle {
     double* loss_part = nullptr;   // [tr_rows]
     double* loss_d = nullptr;
     float *center = nullptr, *half = nullptr;
+    float* x_copy = nullptr;     // [max_batch][NIN]: mlp_forward's inputs where its outputs overlap them
     int* over_budget = nullptr;  // [MAX_BINS]
     int n_bins = 0;
     float ls_lo = 0.f, ls_hi = 1.f;
@@ -941,6 +942,7 @@ lb_status mlp_create(const mlp_config* cfg, void* cuda_stream, mlp_handle** out)
     if (e == cudaSuccess) e = alloc(h, &h->loss_d, 1);
     if (e == cudaSuccess) e = alloc(h, &h->center, NIN);
     if (e == cudaSuccess) e = alloc(h, &h->half, NIN);
+    if (e == cudaSuccess) e = alloc(h, &h->x_copy, (size_t)cfg->max_batch * NIN);
     if (e == cudaSuccess)  // the fused serving kernel keeps activations and weights in shared memory
         e = cudaFuncSetAttribute(serve_fused_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SRV_SMEM);
     if (e == cudaSuccess)  // and so does the fused training kernel
@@ -989,6 +991,14 @@ lb_status mlp_forward(mlp_handle* h, const float* x, int batch, float* out)
 {
     if (!h || !x || !out) return invalid("mlp: NULL handle or buffer");
     if (check_batch(h, batch) != LB_OK) return LB_ERR_INVALID;
+    // blocks write their queries' outputs while others have yet to read their inputs: an
+    // output buffer that overlaps the inputs gets them from a copy
+    const uintptr_t xb = (uintptr_t)x, ob = (uintptr_t)out;
+    const size_t x_bytes = sizeof(float) * NIN * (size_t)batch, out_bytes = sizeof(float) * NOUT * (size_t)batch;
+    if (xb < ob + out_bytes && ob < xb + x_bytes) {
+        if (cudaMemcpyAsync(h->x_copy, x, x_bytes, cudaMemcpyDeviceToDevice, h->stream) != cudaSuccess) return LB_ERR_CUDA;
+        x = h->x_copy;
+    }
     ServeArgs a = inference_args(h, x, batch);
     a.out = out;
     return launch_inference(h, a);
