@@ -868,12 +868,11 @@ static bool capturing(cudaStream_t st)
     return c != cudaStreamCaptureStatusNone;
 }
 
-// Steps of a small lattice: launches of up to 512 steps (one or two milliseconds,
-// so that other streams' kernels get their turn).
+// Steps of a small lattice, in launches of up to patch_max_steps.
 static cudaError_t patch_steps(lb_handle* h, long long n_steps, int* nl)
 {
     for (long long done = 0; done < n_steps;) {
-        int piece = (int)std::min<long long>(n_steps - done, 512);
+        int piece = (int)std::min<long long>(n_steps - done, patch_max_steps(h->patch));
         int first = -1, every = 0;  // first sampled step of this piece
         long long samples = 0;
         if (h->every > 0) {

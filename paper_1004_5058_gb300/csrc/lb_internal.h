@@ -56,6 +56,7 @@ void patch_set_collision(PatchPlan* p, int collision);
 // none, and at most patch_max_samples); their sums are added to acc_prof and
 // acc_wall in the order of a tiled kernel of tile_x columns.
 int patch_max_samples(const PatchPlan* p);
+int patch_max_steps(const PatchPlan* p);  // steps a launch should take at most
 cudaError_t launch_patch_steps(PatchPlan* p, void* src, void* dst, int steps, int first, int every, bool swap, int tile_x,
                                const CellDev* cells, double* acc_prof, double* acc_wall, unsigned* err,
                                cudaStream_t st, int* n_launches);

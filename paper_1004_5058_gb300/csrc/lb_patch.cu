@@ -595,6 +595,17 @@ PatchPlan* patch_create(const Geom& g, int prec, int bc)
 
 int patch_max_samples(const PatchPlan* p) { return p->slots; }
 
+// Steps of about 2 ms, so that other streams' kernels get their turn, and at most 512.
+// us per step measured / by this line: FP32 64^2 3.2 / 3.2, 256^2 6.6 / 6.9; FP64 64^2
+// 11 / 11, 128^2 14 / 20, 256^2 45 / 54, 320^2 75 / 80; MRT rows take up to 1.5 times as
+// long.  A launch costs about 6 us.
+int patch_max_steps(const PatchPlan* p)
+{
+    const double sites = (double)p->g.n_cells * p->g.nx * p->g.ny;
+    const double us = (p->prec == LB_FP64 ? 8.0 + 7e-4 * sites : 3.0 + 6e-5 * sites) * (p->mrt ? 1.5 : 1.0);
+    return (int)std::min(512.0, std::max(1.0, 2000.0 / us));
+}
+
 void patch_set_collision(PatchPlan* p, int collision) { p->mrt = collision == TILED_MRT; }
 
 template <class C, int NS, int DW>
