@@ -70,7 +70,8 @@ typedef enum { LB_FP32 = 0, LB_FP16_SHIFTED = 1, LB_FP64 = 2, LB_FP16_SHIFTED_SR
 /* Kernel family: AUTO picks TILED when the shape allows it, else GENERIC.  Under
  * AUTO lb_step advances a small lattice (below 2^16 sites over all cells, FP64 2^17) with a kernel
  * that takes many steps per launch; the family AUTO picked then serves steps
- * inside a capture of the caller's and is what lb_get_kernel reports. */
+ * inside a capture of the caller's, and all steps on a stream that refuses the
+ * cooperative launch, and is what lb_get_kernel reports. */
 typedef enum { LB_KERNEL_AUTO = 0, LB_KERNEL_GENERIC = 1, LB_KERNEL_TILED = 2 } lb_kernel;
 
 /* One lattice cell, in the paper's symbols.  All cells of a handle share nx, ny
@@ -267,6 +268,10 @@ lb_status lb_load(lb_handle* h, const char* path);
  *              faults: the device stays usable and lb_init_fields recovers.
  *   fault = 2  the step fails at once with LB_ERR_CUDA, as a failed launch
  *              would, without enqueuing anything; the state is unchanged.
+ *   fault = 3  the next launch of the kernel that takes many steps (small lattices
+ *              under LB_KERNEL_AUTO, else LB_ERR_UNSUPPORTED) is refused, as on a
+ *              stream with fewer SMs than its blocks need: that step and the
+ *              later ones run the family of lb_get_kernel.
  *   fault = 0  disarms.  Other values: LB_ERR_INVALID. */
 lb_status lb_test_inject(lb_handle* h, int fault);
 

@@ -72,8 +72,9 @@ struct lb_handle {
     // steps at a time; large ones of a width lb_set_kernel refuses to the tiled kernel
     PatchPlan* patch = nullptr;
     TiledPlan* any_width = nullptr;
+    bool patch_refused = false;  // the stream does not take the patch kernel's cooperative launch
     long long launches = 0;
-    int inject = 0;  // lb_test_inject: 1 = stalled row copy, 2 = failed launch (next lb_step)
+    int inject = 0;  // lb_test_inject: the fault armed for the next lb_step
     std::string last_error;
     // CUDA graphs of step chunks, keyed by (source buffer, steps, sampled last step)
     std::map<std::tuple<int, int, int>, cudaGraphExec_t> graphs;
@@ -282,6 +283,7 @@ static void drop_auto(lb_handle* h)
 {
     patch_destroy(h->patch);
     h->patch = nullptr;
+    h->patch_refused = false;
     if (h->any_width) tiled_destroy(h->any_width);
     h->any_width = nullptr;
 }
@@ -868,11 +870,13 @@ static bool capturing(cudaStream_t st)
     return c != cudaStreamCaptureStatusNone;
 }
 
-// Steps of a small lattice, in launches of up to patch_max_steps.
-static cudaError_t patch_steps(lb_handle* h, long long n_steps, int* nl)
+// Steps of a small lattice, in launches of up to patch_max_steps; *done: those enqueued.
+// *refused: the launch that failed did not take place (a stream with fewer SMs, a
+// partition of the device, than the cooperative grid counts on).
+static cudaError_t patch_steps(lb_handle* h, long long n_steps, long long* done, bool* refused, int* nl)
 {
-    for (long long done = 0; done < n_steps;) {
-        int piece = (int)std::min<long long>(n_steps - done, patch_max_steps(h->patch));
+    while (*done < n_steps) {
+        int piece = (int)std::min<long long>(n_steps - *done, patch_max_steps(h->patch));
         int first = -1, every = 0;  // first sampled step of this piece
         long long samples = 0;
         if (h->every > 0) {
@@ -885,14 +889,21 @@ static cudaError_t patch_steps(lb_handle* h, long long n_steps, int* nl)
                 piece = (int)std::min<long long>(piece, next + samples * every);
             }
         }
-        const cudaError_t e = launch_patch_steps(h->patch, h->f[h->cur], h->f[h->cur ^ 1], piece, first, every, true,
-                                                 h->tile_x, h->d_cells, h->acc_prof, h->acc_wall, h->d_err, h->stream,
-                                                 nl);
-        if (e != cudaSuccess) return e;
+        const int launches = *nl;
+        cudaError_t e = cudaErrorCooperativeLaunchTooLarge;
+        if (h->inject == 3)
+            h->inject = 0;
+        else
+            e = launch_patch_steps(h->patch, h->f[h->cur], h->f[h->cur ^ 1], piece, first, every, true, h->tile_x,
+                                   h->d_cells, h->acc_prof, h->acc_wall, h->d_err, h->stream, nl);
+        if (e != cudaSuccess) {
+            *refused = *nl == launches;
+            return e;
+        }
         h->cur ^= piece & 1;
         h->t += piece;
         h->n_samples += samples;
-        done += piece;
+        *done += piece;
     }
     return cudaSuccess;
 }
@@ -923,13 +934,12 @@ lb_status lb_step(lb_handle* h, long long n_steps)
     }
     int nl = 0;
     long long done = 0;
-    if (h->patch && h->inject != 1 && !capturing(h->stream)) {
-        const cudaError_t e = patch_steps(h, n_steps, &nl);
+    if (h->patch && !h->patch_refused && h->inject != 1 && !capturing(h->stream)) {
+        const cudaError_t e = patch_steps(h, n_steps, &done, &h->patch_refused, &nl);
         if (e != cudaSuccess) {
             cudaGetLastError();
-            return fail(h, LB_ERR_CUDA, "lb_step: launch failed: %s", cudaGetErrorString(e));
-        }
-        done = n_steps;
+            if (!h->patch_refused) return fail(h, LB_ERR_CUDA, "lb_step: launch failed: %s", cudaGetErrorString(e));
+        }  // refused: the rest, and later calls, step by step
     }
     while (done < n_steps) {
         // steps up to and including the next sampled step (or the end)
@@ -1227,9 +1237,11 @@ lb_status lb_autotune(lb_handle* h, const char* cache_path)
 lb_status lb_test_inject(lb_handle* h, int fault)
 {
     if (!h) return LB_ERR_INVALID;
-    if (fault < 0 || fault > 2) return fail(h, LB_ERR_INVALID, "lb_test_inject: unknown fault %d", fault);
+    if (fault < 0 || fault > 3) return fail(h, LB_ERR_INVALID, "lb_test_inject: unknown fault %d", fault);
     if (fault == 1 && h->kernel != LB_KERNEL_TILED)
         return fail(h, LB_ERR_UNSUPPORTED, "lb_test_inject: a stalled copy needs the tiled kernel");
+    if (fault == 3 && !h->patch)
+        return fail(h, LB_ERR_UNSUPPORTED, "lb_test_inject: a refused launch needs the kernel of many steps");
     h->inject = fault;
     return LB_OK;
 }
