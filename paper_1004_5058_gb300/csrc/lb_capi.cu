@@ -919,12 +919,17 @@ lb_status lb_step(lb_handle* h, long long n_steps)
     if (!h->initialised) return fail(h, LB_ERR_STATE, "lb_step: no state loaded (call lb_init_fields)");
     if (h->faulted) return fail(h, LB_ERR_STATE, "lb_step: an earlier device error left the state invalid");
     CK(h, cudaSetDevice(h->device));
-    if (h->batch_pending && cudaEventQuery(h->batch_done) == cudaSuccess) {
-        h->batch_pending = false;
-        if (h->h_err[0]) {
-            h->faulted = true;
-            return fail(h, (h->h_err[0] & ERR_TIMEOUT) ? LB_ERR_TIMEOUT : LB_ERR_NONFINITE,
-                        "lb_step: the previous batch reported a device error (%u)", h->h_err[0]);
+    if (h->batch_pending) {
+        const cudaError_t e = cudaEventQuery(h->batch_done);
+        if (e == cudaSuccess) {
+            h->batch_pending = false;
+            if (h->h_err[0]) {
+                h->faulted = true;
+                return fail(h, (h->h_err[0] & ERR_TIMEOUT) ? LB_ERR_TIMEOUT : LB_ERR_NONFINITE,
+                            "lb_step: the previous batch reported a device error (%u)", h->h_err[0]);
+            }
+        } else if (e != cudaErrorNotReady) {
+            cudaGetLastError();  // an event recorded in a capture has no state: not the next launch's error
         }
     }
     if (n_steps == 0) return LB_OK;

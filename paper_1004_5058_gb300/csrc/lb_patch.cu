@@ -608,22 +608,25 @@ int patch_max_steps(const PatchPlan* p)
 
 void patch_set_collision(PatchPlan* p, int collision) { p->mrt = collision == TILED_MRT; }
 
+// (the launches' own codes: cudaGetLastError would also return an error that an
+// earlier call of the same thread left behind)
 template <class C, int NS, int DW>
-static void launch_patch_finish(const PatchPlan* p, int samples, int tile_x, double* acc_prof, double* acc_wall,
-                                cudaStream_t st)
+static cudaError_t launch_patch_finish(const PatchPlan* p, int samples, int tile_x, double* acc_prof, double* acc_wall,
+                                       cudaStream_t st)
 {
     const Geom& g = p->g;
-    const dim3 grid((g.n_cells * g.ny + 3) / 4);
-    auto go = [&](auto kernel) {
-        kernel<<<grid, 128, 0, st>>>((const C*)p->u, (const C*)p->dp, samples, g.nx, g.ny, g.n_cells, p->bc, acc_prof,
-                                     acc_wall);
-    };
+    const void* k;
     switch (tile_x) {
-    case 64: return go(patch_finish_kernel<C, NS, DW, 2>);
-    case 128: return go(patch_finish_kernel<C, NS, DW, 4>);
-    case 256: return go(patch_finish_kernel<C, NS, DW, 8>);
-    default: return go(patch_finish_kernel<C, NS, DW, 1>);
+    case 64: k = reinterpret_cast<const void*>(&patch_finish_kernel<C, NS, DW, 2>); break;
+    case 128: k = reinterpret_cast<const void*>(&patch_finish_kernel<C, NS, DW, 4>); break;
+    case 256: k = reinterpret_cast<const void*>(&patch_finish_kernel<C, NS, DW, 8>); break;
+    default: k = reinterpret_cast<const void*>(&patch_finish_kernel<C, NS, DW, 1>); break;
     }
+    const C *u = (const C*)p->u, *dp = (const C*)p->dp;
+    int nx = g.nx, ny = g.ny, n_cells = g.n_cells, bc = p->bc;
+    void* args[] = {(void*)&u, (void*)&dp, (void*)&samples, (void*)&nx, (void*)&ny, (void*)&n_cells, (void*)&bc,
+                    (void*)&acc_prof, (void*)&acc_wall};
+    return cudaLaunchKernel(k, dim3((n_cells * ny + 3) / 4), dim3(128), args, 0, st);
 }
 
 cudaError_t launch_patch_steps(PatchPlan* p, void* src, void* dst, int steps, int first, int every, bool swap, int tile_x,
@@ -658,13 +661,11 @@ cudaError_t launch_patch_steps(PatchPlan* p, void* src, void* dst, int steps, in
     if (e != cudaSuccess) return e;
     *n_launches += 1;
     if (samples > 0) {
-        if (p->prec == LB_FP64)
-            launch_patch_finish<double, 1, 3>(p, samples, tile_x, acc_prof, acc_wall, st);
-        else
-            launch_patch_finish<float, 2, 1>(p, samples, tile_x, acc_prof, acc_wall, st);
+        e = p->prec == LB_FP64 ? launch_patch_finish<double, 1, 3>(p, samples, tile_x, acc_prof, acc_wall, st)
+                               : launch_patch_finish<float, 2, 1>(p, samples, tile_x, acc_prof, acc_wall, st);
         *n_launches += 1;
     }
-    return cudaGetLastError();
+    return e;
 }
 
 }  // namespace lbhb
