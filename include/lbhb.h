@@ -272,6 +272,11 @@ lb_status lb_load(lb_handle* h, const char* path);
  *              under LB_KERNEL_AUTO, else LB_ERR_UNSUPPORTED) is refused, as on a
  *              stream with fewer SMs than its blocks need: that step and the
  *              later ones run the family of lb_get_kernel.
+ *   fault = 4  in the next launch of that kernel (of at least two steps) one
+ *              block never announces its first step: the waits for it run out
+ *              after 0.2 s (1.5 s in other launches), every block returns, later
+ *              launches of the batch exit at once, and the next synchronising
+ *              call reports LB_ERR_TIMEOUT, as after fault 1.
  *   fault = 0  disarms.  Other values: LB_ERR_INVALID. */
 lb_status lb_test_inject(lb_handle* h, int fault);
 

@@ -891,6 +891,10 @@ static cudaError_t patch_steps(lb_handle* h, long long n_steps, long long* done,
         }
         const int launches = *nl;
         cudaError_t e = cudaErrorCooperativeLaunchTooLarge;
+        if (h->inject == 4) {
+            h->inject = 0;
+            patch_inject_withhold(h->patch);
+        }
         if (h->inject == 3)
             h->inject = 0;
         else
@@ -1242,11 +1246,11 @@ lb_status lb_autotune(lb_handle* h, const char* cache_path)
 lb_status lb_test_inject(lb_handle* h, int fault)
 {
     if (!h) return LB_ERR_INVALID;
-    if (fault < 0 || fault > 3) return fail(h, LB_ERR_INVALID, "lb_test_inject: unknown fault %d", fault);
+    if (fault < 0 || fault > 4) return fail(h, LB_ERR_INVALID, "lb_test_inject: unknown fault %d", fault);
     if (fault == 1 && h->kernel != LB_KERNEL_TILED)
         return fail(h, LB_ERR_UNSUPPORTED, "lb_test_inject: a stalled copy needs the tiled kernel");
-    if (fault == 3 && !h->patch)
-        return fail(h, LB_ERR_UNSUPPORTED, "lb_test_inject: a refused launch needs the kernel of many steps");
+    if (fault >= 3 && (!h->patch || h->patch_refused))
+        return fail(h, LB_ERR_UNSUPPORTED, "lb_test_inject: fault %d needs the kernel of many steps", fault);
     h->inject = fault;
     return LB_OK;
 }

@@ -50,6 +50,9 @@ struct PatchPlan;
 PatchPlan* patch_create(const Geom& g, int prec, int bc);
 void patch_destroy(PatchPlan* p);
 void patch_set_collision(PatchPlan* p, int collision);
+// Failure injection (tests): the next launch leaves one flag unset, so the waits for
+// it run out (after 0.2 s).
+void patch_inject_withhold(PatchPlan* p);
 // `steps` steps from src, ping-ponging with dst (swap), or reading src and writing
 // dst every time (timing a kernel without changing the state).  Sampled steps:
 // first, first + every, ... counted from this launch's first step (first < 0:

@@ -56,6 +56,8 @@ struct PatchArgs {
     void *u, *dp;
     unsigned* err;
     unsigned* flags;  // [cell][npy][npx] steps done
+    unsigned long long wait_ns;  // bound of each wait for a flag
+    unsigned withhold;           // failure injection (tests): patch 0 never sets its flag
 };
 
 // Pair p, p + 1 of stored elements through L2 (the data other blocks of this
@@ -144,15 +146,14 @@ __device__ __forceinline__ void st_release(unsigned* p, unsigned v)
 {
     asm volatile("st.release.gpu.global.u32 [%0], %1;" ::"l"(p), "r"(v) : "memory");
 }
-// Waits until *p has reached v, for at most 1.5 s of wall time (a step takes
-// microseconds); false when the time ran out.
-__device__ __noinline__ bool wait_flag_bounded(const unsigned* p, unsigned v)
+// Waits until *p has reached v, for at most `ns` of wall time; false when the time ran out.
+__device__ __noinline__ bool wait_flag_bounded(const unsigned* p, unsigned v, unsigned long long ns)
 {
     if ((int)(ld_acquire(p) - v) >= 0) return true;
     const uint64_t t0 = global_ns();
     for (uint32_t it = 1;; ++it) {
         if ((int)(ld_acquire(p) - v) >= 0) return true;
-        if ((it & 63u) == 0 && global_ns() - t0 > 1500000000ull) return false;
+        if ((it & 63u) == 0 && global_ns() - t0 > ns) return false;
     }
 }
 
@@ -218,7 +219,7 @@ __global__ void __launch_bounds__(PATCH_THREADS) patch_steps_kernel(const __grid
                     const int qx = column(i < 2 ? x0 - 3 + 2 * i : (i == 2 ? x0 : ex + 2 * i - 5), nx);
                     int qy = j < 2 ? y0 - 3 + 2 * j : (j == 2 ? y0 : ey + 2 * j - 5);
                     qy = a.bc == 0 ? column(qy, ny) : min(max(qy, 0), ny - 1);
-                    late = !wait_flag_bounded(a.flags + (cell * a.npy + qy / BY) * a.npx + qx / BX, (unsigned)s);
+                    late = !wait_flag_bounded(a.flags + (cell * a.npy + qy / BY) * a.npx + qx / BX, (unsigned)s, a.wait_ns);
                 }
                 if (__syncthreads_or(late)) {
                     if (t == 0) atomicOr(a.err, ERR_TIMEOUT);
@@ -420,7 +421,7 @@ __global__ void __launch_bounds__(PATCH_THREADS) patch_steps_kernel(const __grid
             }
             // every thread is done with shared memory and has stored its pair
             __syncthreads();
-            if (t == 0 && a.steps > 1) st_release(a.flags + p, (unsigned)(s + 1));
+            if (t == 0 && a.steps > 1 && p >= (int)a.withhold) st_release(a.flags + p, (unsigned)(s + 1));
             cell += d_cell;
             py += d_py;
             px += d_px;
@@ -499,6 +500,7 @@ struct PatchPlan {
     size_t smem;
     int mrt = 0;
     int slots;  // sampled steps a launch may hold
+    bool withhold = false;  // failure injection for the next launch (tests)
     void* mem = nullptr;  // one allocation: the sampled steps' values and the flags
     void *u, *dp;
     unsigned* flags;
@@ -606,6 +608,8 @@ int patch_max_steps(const PatchPlan* p)
     return (int)std::min(512.0, std::max(1.0, 2000.0 / us));
 }
 
+void patch_inject_withhold(PatchPlan* p) { p->withhold = true; }
+
 void patch_set_collision(PatchPlan* p, int collision) { p->mrt = collision == TILED_MRT; }
 
 // (the launches' own codes: cudaGetLastError would also return an error that an
@@ -653,6 +657,9 @@ cudaError_t launch_patch_steps(PatchPlan* p, void* src, void* dst, int steps, in
     a.dp = p->dp;
     a.err = err;
     a.flags = p->flags;
+    a.wait_ns = p->withhold ? 200000000ull : 1500000000ull;  // a step takes microseconds
+    a.withhold = p->withhold ? 1u : 0u;
+    p->withhold = false;  // one launch only
     if (steps > 1) e = cudaMemsetAsync(p->flags, 0, sizeof(unsigned) * p->g.n_cells * p->npx * p->npy, st);
     if (e != cudaSuccess) return e;
     void* args[] = {(void*)&a};
