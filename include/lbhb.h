@@ -261,7 +261,8 @@ lb_status lb_load(lb_handle* h, const char* path);
 /* Test hook for the failure paths (the paper has no counterpart): arms one
  * fault for the next lb_step of this handle.
  *   fault = 1  the first launch of that step leaves one row copy of its first
- *              CTA unissued (tiled kernel only, else LB_ERR_UNSUPPORTED): the
+ *              CTA unissued (tiled kernel only, its any-width form included, else
+ *              LB_ERR_UNSUPPORTED): the
  *              waits for it run out after their 1.5 s bound, the kernel records
  *              a timeout and returns, later launches of the batch exit at once,
  *              and the next synchronising call reports LB_ERR_TIMEOUT.  Nothing

@@ -971,13 +971,13 @@ lb_status lb_step(lb_handle* h, long long n_steps)
         while (chunk > 0) {
             const long long piece_max = 64;
             // an injected stall applies to one plain launch, never to a captured graph
-            const bool stall = h->inject == 1 && h->plan != nullptr;
+            const bool stall = h->inject == 1 && step_plan(h) != nullptr;
             const long long piece = stall ? 1 : (chunk > piece_max ? piece_max : chunk);
             const bool s_last = sample_last && piece == chunk;
             cudaError_t e;
             if (stall) {
                 h->inject = 0;
-                tiled_inject_skip(h->plan, 5);
+                tiled_inject_skip(step_plan(h), 5);
                 e = enqueue_one_step(h, h->cur, s_last, &nl);
             } else {
                 e = run_chunk(h, h->cur, (int)piece, s_last, &nl);
@@ -1247,7 +1247,7 @@ lb_status lb_test_inject(lb_handle* h, int fault)
 {
     if (!h) return LB_ERR_INVALID;
     if (fault < 0 || fault > 4) return fail(h, LB_ERR_INVALID, "lb_test_inject: unknown fault %d", fault);
-    if (fault == 1 && h->kernel != LB_KERNEL_TILED)
+    if (fault == 1 && !step_plan(h))
         return fail(h, LB_ERR_UNSUPPORTED, "lb_test_inject: a stalled copy needs the tiled kernel");
     if (fault >= 3 && (!h->patch || h->patch_refused))
         return fail(h, LB_ERR_UNSUPPORTED, "lb_test_inject: fault %d needs the kernel of many steps", fault);
