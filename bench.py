@@ -46,8 +46,8 @@ FALLBACK_HBM_GBS = 6800.0
 # kernel at tau = 1, the workload's: dfma 93, dadd 118, dmul 48 per site; each
 # occupies the pipe once) against the pipe's rate, 152 SMs x 2 FP64 operations
 # per clock (the nominal 1.25 TFLOP/s of FMA at the 2070 MHz maximum SM clock),
-# at the SM clock sampled in the run.  The count is the tiled kernel's; for the
-# generic kernel pair the line reports no FP64 roofline.
+# at the SM clock sampled in the run.  The count is the tiled kernel's; where
+# another kernel steps (step_form) the line reports no FP64 roofline.
 FP64_OPS_PER_SITE = 93 + 118 + 48
 FP64_OPS_PER_CLOCK, N_SM, SM_MAX_MHZ = 2, 152, 2070.0
 
@@ -355,7 +355,7 @@ def batched_vs_plain(args, torch, Lattice, hb_fit):
     with Lattice(cells, args.precision) as lat:
         lat.init_fields(ra, rb, ux, uy)
         lat.autotune(cache)
-        kern_b = lat.kernel()
+        kern_b, form_b = lat.kernel(), lat.step_form()
         sweep(lat, slice(0, n))  # the graphs of this step pattern, untimed
         torch.cuda.synchronize()
         t0 = time.perf_counter()
@@ -363,7 +363,7 @@ def batched_vs_plain(args, torch, Lattice, hb_fit):
         wall_b = time.perf_counter() - t0
     lats = [Lattice([c], args.precision) for c in cells]
     try:
-        kern_p = lats[0].kernel()
+        kern_p, form_p = lats[0].kernel(), lats[0].step_form()
         sig_p, S_p, dev_p = np.empty(n), np.empty(n), 0.0
         torch.cuda.synchronize()
         t0 = time.perf_counter()
@@ -386,9 +386,9 @@ def batched_vs_plain(args, torch, Lattice, hb_fit):
                     "%s, %d time steps, second half sampled every %d" % (args.precision.upper(), steps, every),
         "cells": n, "steps": steps,
         "batched": {"mlups": sites * steps / dev_b / 1e6, "wall_s": wall_b, "points_per_s": n / wall_b,
-                    "kernel": list(kern_b)},
+                    "kernel": list(kern_b), "step_form": form_b},
         "plain": {"mlups": sites * steps / dev_p / 1e6, "wall_s": wall_p, "points_per_s": n / wall_p,
-                  "kernel": list(kern_p)},
+                  "kernel": list(kern_p), "step_form": form_p},
         "speedup_wall": wall_p / wall_b, "speedup_device": dev_p / dev_b,
         "sigma_max_rel_diff": float(np.max(rel)), "sigma_bitwise_equal": bool(np.array_equal(sig_b, sig_p)),
         "hb_fit_batched": fits,
@@ -424,7 +424,9 @@ def run_ours(args):
         cache_dir = os.path.join(ROOT, "paper_1004_5058_gb300", "_build")  # the library's build folder
         lat.autotune(os.path.join(cache_dir, "autotune_cache.txt") if os.path.isdir(cache_dir) else None)
     kernel, tx, ty = lat.kernel()
-    shape = lat.launch_shape()
+    form = lat.step_form()
+    tiled = form == "tiled"  # what is known of the tiled kernel's launches holds for no other kernel
+    shape = lat.launch_shape() if tiled else None
     launch_shape = None if shape is None else dict(zip(("ctas", "ctas_sampled", "threads", "smem_bytes"), shape))
     stream = torch.cuda.ExternalStream(lat.stream_ptr)
     lat.set_sampling(0, args.every)
@@ -488,14 +490,15 @@ def run_ours(args):
     predicted_ms = 1e3 * ((chunk - n_sampled_per_step) * t_plain + n_sampled_per_step * t_sampled)
     alg_bytes = BYTES_PER_SITE[args.precision] * sites
     peak, peak_kind = peaks()
-    achieved = alg_bytes / (t_launch if kernels_per_step == 1 else t_launch * kernels_per_step) / 1e9
+    achieved = alg_bytes / t_plain / 1e9
     traffic = (committed_traffic(args.precision, nx, ny, n_cells, two_time=args.tau_b not in (0.0, 1.0),
-                                 mrt=bool(args.mrt)) if kernel == "tiled" else None)
+                                 mrt=bool(args.mrt)) if tiled else None)
 
     roofline = {"bound": "hbm", "achieved": achieved, "peak": peak, "unit": "GB/s",
                 "frac": achieved / peak, "traffic": traffic,
                 "peak_source": "%s copy bandwidth" % peak_kind,
-                "algorithmic_bytes_per_launch": alg_bytes, "mean_launch_ms": t_launch * 1e3,
+                "algorithmic_bytes_per_launch": alg_bytes / kernels_per_step, "steps_per_launch": 1.0 / kernels_per_step,
+                "mean_launch_ms": t_launch * 1e3,
                 "bytes_per_site_update": BYTES_PER_SITE[args.precision],
                 "launches_timed": n_roof,
                 # the timed region reconciled from separately timed plain and sampled steps
@@ -505,12 +508,13 @@ def run_ours(args):
         sm_mhz = (clk or {}).get("sm_mhz") or SM_MAX_MHZ
         p64 = N_SM * FP64_OPS_PER_CLOCK * sm_mhz * 1e-3
         # the op count is the BGK kernel's (the MRT one adds its correction)
-        gops = FP64_OPS_PER_SITE * sites / t_plain / 1e9 if kernel == "tiled" and not args.mrt else None
+        gops = FP64_OPS_PER_SITE * sites / t_plain / 1e9 if tiled and not args.mrt else None
         roofline = {"bound": "alu", "achieved": gops, "peak": p64, "unit": "G FP64 op/s",
-                    "frac": None if gops is None else gops / p64, "kernel": kernel,
+                    "frac": None if gops is None else gops / p64, "kernel": kernel, "step_form": form,
                     "traffic": traffic,
                     "peak_source": "FP64 pipe: 152 SMs x 2 ops per clock at the sampled SM clock (%.0f MHz)" % sm_mhz,
                     "fp64_ops_per_site_update": FP64_OPS_PER_SITE, "mean_launch_ms": t_launch * 1e3,
+                    "steps_per_launch": 1.0 / kernels_per_step,
                     "hbm": {"achieved": achieved, "peak": peak, "unit": "GB/s", "frac": achieved / peak}}
 
     # end to end through the C ABI with host buffers
@@ -580,7 +584,7 @@ def run_ours(args):
         "vs_baseline": None, "dtype": {"fp32": "f32", "fp16": "f16-storage/f32", "fp16sr": "f16-storage/f32",
                                        "fp64": "f64"}[args.precision],
         "data": "synthetic",
-        "config": dict(workload_config(args), kernel=kernel, tile=[tx, ty], launch=launch_shape),
+        "config": dict(workload_config(args), kernel=kernel, step_form=form, tile=[tx, ty], launch=launch_shape),
         "roofline": roofline,
         "e2e": {"value": e2e_value, "unit": UNIT, "h2d_bytes_per_step": h2d, "d2h_bytes_per_step": d2h,
                 "lattice_steps_per_step": chunk, "steps": e2e_steps,

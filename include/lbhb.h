@@ -67,11 +67,13 @@ typedef enum { LB_BC_PERIODIC = 0, LB_BC_COUETTE = 1 } lb_bc;
  * Observables are reduced in FP64. */
 typedef enum { LB_FP32 = 0, LB_FP16_SHIFTED = 1, LB_FP64 = 2, LB_FP16_SHIFTED_SR = 3 } lb_precision;
 
-/* Kernel family: AUTO picks TILED when the shape allows it, else GENERIC.  Under
- * AUTO lb_step advances a small lattice (below 2^16 sites over all cells, FP64 2^17) with a kernel
- * that takes many steps per launch; the family AUTO picked then serves steps
- * inside a capture of the caller's, and all steps on a stream that refuses the
- * cooperative launch, and is what lb_get_kernel reports. */
+/* Kernel family: AUTO picks TILED when the shape allows it, else GENERIC, and that
+ * is what lb_get_kernel reports.  Under AUTO lb_step advances a small lattice (below
+ * 2^16 sites over all cells, FP64 2^17; FP16 only where the tiled kernel takes the
+ * width) with a kernel that takes many steps per launch; the family AUTO picked then
+ * serves steps inside a capture of the caller's, and all steps on a stream that
+ * refuses the cooperative launch.  Larger FP32 lattices of a width the tiled kernel
+ * does not take run its any-width form.  lb_get_step_form tells which kernel steps. */
 typedef enum { LB_KERNEL_AUTO = 0, LB_KERNEL_GENERIC = 1, LB_KERNEL_TILED = 2 } lb_kernel;
 
 /* One lattice cell, in the paper's symbols.  All cells of a handle share nx, ny
@@ -222,13 +224,26 @@ lb_status lb_set_kernel(lb_handle* h, lb_kernel kernel, int tile_x, int tile_y);
  * precision.  Synchronous. */
 lb_status lb_autotune(lb_handle* h, const char* cache_path);
 
-/* Reads the kernel family and tile in use (outputs nullable). */
+/* Reads the kernel family and tile in use (outputs nullable).  Under
+ * LB_KERNEL_AUTO lb_step may run another kernel in its place: lb_get_step_form. */
 lb_status lb_get_kernel(const lb_handle* h, lb_kernel* kernel, int* tile_x, int* tile_y);
 
-/* Launch shape of the tiled kernel in use (outputs nullable): persistent CTAs of
- * plain and of sampled steps (each as many as fit on the GPU, at most one per
- * work item), threads and dynamic shared memory bytes per CTA.
- * LB_ERR_UNSUPPORTED for the generic kernel. */
+/* What lb_step runs outside a capture of the caller's:
+ *   LB_STEP_GENERIC    the generic pair, two launches per step
+ *   LB_STEP_TILED      the tiled kernel with the tile of lb_get_kernel
+ *   LB_STEP_TILED_ANY  the tiled kernel's any-width form, with a tile of its own
+ *                      (AUTO, larger FP32 lattices of a width that lb_set_kernel
+ *                      refuses to the tiled kernel; lb_get_kernel says GENERIC)
+ *   LB_STEP_PATCH      the kernel that takes many steps per launch (AUTO, small
+ *                      lattices; lb_get_kernel says what a captured step runs) */
+typedef enum { LB_STEP_GENERIC = 1, LB_STEP_TILED = 2, LB_STEP_TILED_ANY = 3, LB_STEP_PATCH = 4 } lb_step_form;
+lb_status lb_get_step_form(const lb_handle* h, lb_step_form* form);
+
+/* Launch shape of the tiled kernel of lb_get_kernel (outputs nullable): persistent
+ * CTAs of plain and of sampled steps (each as many as fit on the GPU, at most one
+ * per work item), threads and dynamic shared memory bytes per CTA.  These are the
+ * launches of lb_step where lb_get_step_form says LB_STEP_TILED.
+ * LB_ERR_UNSUPPORTED where lb_get_kernel says GENERIC. */
 lb_status lb_launch_shape(const lb_handle* h, int* ctas, int* ctas_sampled, int* threads, int* smem_bytes);
 
 /* Waits for all enqueued work of the handle; reports device errors. */

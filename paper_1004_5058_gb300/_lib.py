@@ -73,6 +73,7 @@ SIGNATURES = {
     "lb_slab_get": (C.c_int, [_H, C.c_int, C.c_void_p]),
     "lb_slab_put": (C.c_int, [_H, C.c_int, C.c_void_p]),
     "lb_wall_momentum": (C.c_int, [_H, _D, C.POINTER(C.c_longlong)]),
+    "lb_get_step_form": (C.c_int, [_H, C.POINTER(C.c_int)]),
     "lb_launch_shape": (C.c_int, [_H, C.POINTER(C.c_int), C.POINTER(C.c_int), C.POINTER(C.c_int),
                                   C.POINTER(C.c_int)]),
     # include/lbhb_mlp.h

@@ -1142,6 +1142,16 @@ lb_status lb_get_kernel(const lb_handle* h, lb_kernel* kernel, int* tile_x, int*
     return LB_OK;
 }
 
+lb_status lb_get_step_form(const lb_handle* h, lb_step_form* form)
+{
+    if (!h || !form) return LB_ERR_INVALID;
+    *form = h->patch && !h->patch_refused    ? LB_STEP_PATCH
+            : h->kernel == LB_KERNEL_TILED ? LB_STEP_TILED
+            : h->any_width                 ? LB_STEP_TILED_ANY
+                                           : LB_STEP_GENERIC;
+    return LB_OK;
+}
+
 lb_status lb_launch_shape(const lb_handle* h, int* ctas, int* ctas_sampled, int* threads, int* smem_bytes)
 {
     if (!h) return LB_ERR_INVALID;

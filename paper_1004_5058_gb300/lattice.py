@@ -17,6 +17,7 @@ PRECISIONS = {"fp32": L.LB_FP32, "fp16": L.LB_FP16_SHIFTED, "fp16_shifted": L.LB
               "fp16sr": L.LB_FP16_SHIFTED_SR}
 KERNELS = {"auto": L.LB_KERNEL_AUTO, "generic": L.LB_KERNEL_GENERIC, "tiled": L.LB_KERNEL_TILED}
 KERNEL_NAMES = {v: k for k, v in KERNELS.items()}
+STEP_FORMS = {1: "generic", 2: "tiled", 3: "tiled any width", 4: "patch"}  # lb_step_form
 
 
 def _dp(a):
@@ -209,9 +210,17 @@ class Lattice:
         self._chk(self.lib.lb_get_kernel(self.h, C.byref(k), C.byref(tx), C.byref(ty)))
         return KERNEL_NAMES[k.value], tx.value, ty.value
 
+    def step_form(self) -> str:
+        """The kernel that step() runs: "generic", "tiled", "tiled any width" or
+        "patch" (many steps per launch); lb_get_step_form."""
+        v = C.c_int()
+        self._chk(self.lib.lb_get_step_form(self.h, C.byref(v)))
+        return STEP_FORMS[v.value]
+
     def launch_shape(self):
         """(CTAs of plain steps, CTAs of sampled steps, threads, shared memory
-        bytes) of the tiled kernel in use, or None for the generic kernel."""
+        bytes) of the tiled kernel of kernel(), or None for the generic kernel;
+        step() launches it so where step_form() is "tiled"."""
         v = [C.c_int() for _ in range(4)]
         st = self.lib.lb_launch_shape(self.h, *[C.byref(x) for x in v])
         if st == L.LB_ERR_UNSUPPORTED:

@@ -61,14 +61,14 @@ def precision_study(n: int = 4096, u_wall: float = 1e-3, steps: int = 50000, eve
             sigma, S, Sb = lat.shear_stress()
             mass, _ = lat.reductions()
             res[prec] = dict(rho_a=a[0], rho_b=b[0], sigma=float(sigma[0]), S=float(S[0]), S_bulk=float(Sb[0]),
-                             mlups=n * n * steps / dt / 1e6, seconds=dt, kernel=lat.kernel(),
+                             mlups=n * n * steps / dt / 1e6, seconds=dt, kernel=lat.kernel(), step_form=lat.step_form(),
                              mass_drift=float(abs(mass[0, 0] - ra.sum()) / ra.sum()),
                              mass_drift_b=float(abs(mass[0, 1] - rb.sum()) / rb.sum()))
     ref = res.get("fp64")
     summary = {"n": n, "u_wall": u_wall, "steps": steps, "g_ab": g_ab}
     for prec, r in res.items():
         row = {"mlups": r["mlups"], "seconds": r["seconds"], "sigma_xy": r["sigma"], "shear_rate": r["S"],
-               "kernel": r["kernel"], "mass_drift": r["mass_drift"], "mass_drift_b": r["mass_drift_b"]}
+               "kernel": r["kernel"], "step_form": r["step_form"], "mass_drift": r["mass_drift"], "mass_drift_b": r["mass_drift_b"]}
         if ref is not None and prec != "fp64":
             row["max_abs_drho"] = float(max(np.abs(r["rho_a"] - ref["rho_a"]).max(),
                                             np.abs(r["rho_b"] - ref["rho_b"]).max()))
@@ -410,7 +410,7 @@ def slab_throughput(n: int = 4096, steps: int = 400, worlds=(2, 4, 8), precision
         lat.init_fields(*fields)
         dt = timed(lambda k: lat.step(k))
         whole = lat.get_populations()[0]
-        out["whole"] = {"seconds": dt, "mlups": n * n * steps / dt / 1e6, "kernel": lat.kernel()}
+        out["whole"] = {"seconds": dt, "mlups": n * n * steps / dt / 1e6, "kernel": lat.kernel(), "step_form": lat.step_form()}
     for world in worlds:
         parts = split_rows(n, world)
         slabs = [SlabLattice([cell], y0, rows, precision, stream=stream) for y0, rows in parts]
