@@ -98,7 +98,8 @@ __device__ __noinline__ void profile_row_sums(const C* ub, int lane, double* __r
 //   FAM_FULL  every strip is TX columns wide (nx a multiple of TX) and every cell
 //             has one relaxation time (BGK);
 //   FAM_FULL_BIG  the same, for lattices far larger than the L2 (full_big): ring rows
-//             are computed per row instead of kept, stores without the streaming hint;
+//             are computed per row instead of kept, stores without the streaming hint,
+//             1/rho and psi/rho by the fast division;
 //   FAM_GEN   the last strip may be narrower (its extra columns masked) and the
 //             species may relax with times of their own (BGK);
 //   FAM_MRT   as FAM_GEN, with the multiple-relaxation-time collision;
@@ -131,6 +132,7 @@ __global__ void __launch_bounds__(tiled_threads(TX),
     // 1024^2 MRT 216.4 -> 209.6 us, 48 x 64^2 10.5 -> 10.3, 1021 x 509 18.4 -> 18.0;
     // FP16, at its register limit, loses 1.5 %, and so does the memory-bound FAM_FULL_BIG
     constexpr bool KEEP = std::is_same<T, float>::value && FAM != FAM_FULL_BIG;
+    constexpr bool DIV = FAM == FAM_FULL_BIG;  // rho_rcp, psi_over_rho
     // stored populations are scale * g (scale 1 except for the dithered FP16 storage)
     constexpr C scale = C(Store<T>::scale), inv_scale = C(1) / scale;
     constexpr int E = (int)sizeof(T);
@@ -446,7 +448,7 @@ __global__ void __launch_bounds__(tiled_threads(TX),
                 jwx = jwx * V(inv_scale);
                 jwy = jwy * V(inv_scale);
             }
-            const V inv_rho = lane_rcp(rho_w);
+            const V inv_rho = rho_rcp<DIV>(rho_w);
             const V ux = jwx * inv_rho, uy = jwy * inv_rho;
             const C fx_body = body_force_x<C>(p, gy);
             const bool body_raw = !one_time && !is_zero(fx_body);  // the force needs the raw 1/rho
@@ -469,11 +471,9 @@ __global__ void __launch_bounds__(tiled_threads(TX),
                     collide_species_shifted<V, false>(f, rho_s, rho_bar2, v[2][1], ux, uy, ax, pu, tau2, ntau2, omega2, fs, &Fx, V(scale));
             } else {
                 if (unit_omega)
-                    collide_species<V, true>(f, rho_s, v[2][1], ux, uy, ax, pu, tau2, ntau2, omega2, fs,
-                                             &Fx);
+                    collide_species<V, true, false, DIV>(f, rho_s, v[2][1], ux, uy, ax, pu, tau2, ntau2, omega2, fs, &Fx);
                 else
-                    collide_species<V, false>(f, rho_s, v[2][1], ux, uy, ax, pu, tau2, ntau2, omega2, fs,
-                                              &Fx);
+                    collide_species<V, false, false, DIV>(f, rho_s, v[2][1], ux, uy, ax, pu, tau2, ntau2, omega2, fs, &Fx);
             }
 
             // stochastic rounding: one stream per thread and row, seeded from the
