@@ -267,13 +267,19 @@ static lb_status select_kernel(lb_handle* h, lb_kernel k, int tx, int ty);
 // The kernel family and tile of LB_KERNEL_AUTO.
 static lb_status select_by_shape(lb_handle* h)
 {
-    // 128 or 64 columns where they divide nx, else the widest tile that fits (a
-    // narrower last strip), else the generic kernel.  32 columns are left to lattices
-    // narrower than 64: us per step 352^2 FP32 9.8 (32) / 8.4 (128), 200^2 FP64 106 / 46
-    const int txs[] = {128, 64, 32};
+    // the widest tile that divides nx, else the widest that fits (a narrower last
+    // strip), else the generic kernel.  In FP32 and FP16 32 columns are left to lattices
+    // narrower than 64: us per step, 32 columns / the widest that fits, FP32 352^2 9.8 /
+    // 8.4, 40 x (96 x 64) 15.5 / 14.1, 16 x (160 x 512) 51.6 / 51.0, 16 x (352 x 512) 106 /
+    // 76.  FP64 rows cost what their warps occupy of the FP64 pipe, masked columns
+    // included: 32 / 64 / 128 columns, 4 x (96 x 512) 135 / 165, 12 x (160 x 300) 345 /
+    // 428 / 663, 12 x (224 x 300) 486 / 559 / 665, 12 x (352 x 300) 771 / 832 / 766; over
+    // 37 shapes of such widths 32 columns take 2 % more than the best of the three (10 %
+    // at most), 64 8 % (33 %), 128 14 % (92 %).
+    const int txs[] = {128, 64, 32}, narrowest = h->prec == LB_FP64 ? 32 : 64;
     for (int pass = 0; pass < 2; ++pass)
         for (int c : txs)
-            if ((pass == 1 || (c > 32 && h->nx % c == 0)) && tiled_supported(h->gbuf, h->elem, c, 0) &&
+            if ((pass == 1 || (c >= narrowest && h->nx % c == 0)) && tiled_supported(h->gbuf, h->elem, c, 0) &&
                 select_kernel(h, LB_KERNEL_TILED, c, 0) == LB_OK)
                 return LB_OK;
     return select_kernel(h, LB_KERNEL_GENERIC, 0, 0);

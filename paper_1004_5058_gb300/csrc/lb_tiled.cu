@@ -73,14 +73,28 @@ static size_t smem_bytes(int tx, int elem, int depth)
 }
 static_assert(tiled_smem_bytes(128, 4) == 74032, "shared memory of the FP32 128-column tile");
 
+// FP64: row times of an SM with `per_sm` work items of ty rows (the four halo rows only
+// pass through psi: 2 rows' worth).  As many items at a time as the SM holds CTAs; a row
+// of theirs takes the FP64 pipes of its four sub-partitions in turn, or one warp's time
+// on one of them where fewer than four column warps run, and one CTA alone leaves the
+// pipe idle for an eighth of the time.  Counting every row as if it filled the pipe gave
+// 12 x (160 x 300) in 32 columns 60-row segments, two warps on an SM, and 565 us per
+// step; 30-row ones take 345.  2 x (480 x 1000) 929 -> 564, 24 x (96 x 96) 231 -> 146.
+static double fp64_row_times(long long per_sm, int ty, int tile_x)
+{
+    const int occ = tiled_min_ctas(tile_x, 8);
+    double t = 0.0;
+    for (long long left = per_sm; left > 0; left -= occ)
+        t += (ty + 2) * std::max(1.0, (double)std::min<long long>(left, occ) * (tile_x / 32) / 4.0);
+    return per_sm == 1 ? 1.13 * t : t;
+}
+
 // Segment height from a model of the time of a launch: work items = strips x
 // segments x cells; an item walks its rows, four halo rows and about 1.5 row-times
 // of start-up one after another, and a row takes longer the more column warps share
 // the SM.  us per row measured on 384^2 .. 1024^2 FP32 cells: 0.75 with one
 // 128-column CTA per SM, 0.93 with two, 1.2 with three (a service warp counts half).  More items than resident
-// CTAs run in rounds.  FP64 rows share the SM's FP64 pipe, so the fullest SM's rows
-// add up (halo rows only pass through psi: 2 for the four), and one CTA alone leaves
-// the pipe idle for an eighth of the time.
+// CTAs run in rounds.  FP64 rows share the SM's FP64 pipe: see fp64_row_times.
 // Heights below 8 (the least before) pay on lattices that do not fill the chip: us
 // per step at 8 rows / at the model's choice: 512^2 FP32 12.3 / 10.8 (5 rows), 48
 // cells of 64^2 12.3 / 10.6 (6), 512^2 FP16 13.5 / 11.9 (5), FP64 177 / 161 (14).
@@ -96,7 +110,7 @@ static int pick_segment_rows(const Geom& g, int nrows, int tile_x, int elem, int
         const long long per_sm = (items + sms - 1) / sms;  // items of the fullest SM
         double cost;
         if (elem == 8) {
-            cost = (double)per_sm * (ty + 2) * (per_sm == 1 ? 1.13 : 1.0);
+            cost = fp64_row_times(per_sm, ty, tile_x);
         } else {
             const long long rounds = (items + (long long)sms * occ - 1) / ((long long)sms * occ);
             const double warps = (double)std::min<long long>(per_sm, occ) * (tile_x / 32 + 0.5);
