@@ -321,8 +321,8 @@ static void select_beyond_family(lb_handle* h)
     } else if (h->kernel == LB_KERNEL_GENERIC) {
         const int tx = h->nx >= 128 ? 128 : 64;
         if (tiled_any_supported(h->gbuf, h->elem, tx))
-            h->any_width = tiled_create(h->gbuf, h->rm, (int)h->prec, h->elem, h->bc, h->f[0], h->f[1], tx, 0, true, nullptr);
-        if (h->any_width) tiled_set_collision(h->any_width, collision_kind(h->cells));
+            h->any_width = tiled_create(h->gbuf, h->rm, (int)h->prec, h->elem, h->bc, h->f[0], h->f[1], tx, 0, true,
+                                        collision_kind(h->cells), nullptr);
     }
 }
 
@@ -362,9 +362,9 @@ static lb_status select_kernel(lb_handle* h, lb_kernel k, int tx, int ty)
     if (tiled_partials_nbx(h->g, tx) > h->nbx_alloc)
         return fail(h, LB_ERR_UNSUPPORTED, "lb_set_kernel: tile %d too narrow for the partial buffers", tx);
     const char* msg = nullptr;
-    TiledPlan* p = tiled_create(h->gbuf, h->rm, (int)h->prec, h->elem, h->bc, h->f[0], h->f[1], tx, ty, false, &msg);
+    TiledPlan* p = tiled_create(h->gbuf, h->rm, (int)h->prec, h->elem, h->bc, h->f[0], h->f[1], tx, ty, false,
+                                collision_kind(h->cells), &msg);
     if (!p) return fail(h, LB_ERR_UNSUPPORTED, "lb_set_kernel: %s", msg ? msg : "tiled plan failed");
-    tiled_set_collision(p, collision_kind(h->cells));
     if (h->plan) tiled_destroy(h->plan);
     drop_auto(h);
     h->plan = p;

@@ -24,7 +24,7 @@ int tiled_partials_nbx(const Geom& g, int tile_x);
 // g: the whole population buffer; rm: the rows a step updates (a whole cell, or
 // the own rows of a slab between its ghost rows).
 TiledPlan* tiled_create(const Geom& g, const RowMap& rm, int prec, int elem_bytes, int bc, void* f0, void* f1,
-                        int tile_x, int tile_y, bool any, const char** err_msg);
+                        int tile_x, int tile_y, bool any, int collision, const char** err_msg);
 void tiled_destroy(TiledPlan* p);
 template <class T>
 cudaError_t launch_tiled_step(TiledPlan* p, int src_buf, const CellDev* cells, bool sample, double* prof_part,

@@ -197,7 +197,7 @@ static bool encode(CUtensorMap* m, void* base, const Geom& g, int elem, int box_
 }
 
 TiledPlan* tiled_create(const Geom& g, const RowMap& rm, int prec, int elem, int bc, void* f0, void* f1, int tile_x,
-                        int tile_y, bool any, const char** err_msg)
+                        int tile_y, bool any, int collision, const char** err_msg)
 {
     if (any ? !tiled_any_supported(g, elem, tile_x) : !tiled_supported(g, elem, tile_x, tile_y)) {
         if (err_msg) *err_msg = "shape/tile not supported by the tiled kernel";
@@ -209,6 +209,7 @@ TiledPlan* tiled_create(const Geom& g, const RowMap& rm, int prec, int elem, int
     p->elem = elem;
     p->bc = bc;
     p->any = any;
+    p->collision = collision;
     p->tx = tile_x;
     p->ty = tile_y;
     p->big = full_big(g, prec, tile_x);
@@ -260,9 +261,11 @@ TiledPlan* tiled_create(const Geom& g, const RowMap& rm, int prec, int elem, int
         }
         occ[fam][smp] = o;
     }
-    // segment height for the plain kernel of the family that will run most
-    if (p->ty <= 0)
-        p->ty = pick_segment_rows(g, rm.nown, tile_x, elem, sms, occ[any ? FAM_ANY : full_ok ? full : FAM_GEN][0]);
+    // segment height for the plain kernel of the family that these cells run: by the BGK
+    // kernel's CTAs per SM, which the MRT kernel's registers do not allow in 64 columns,
+    // MRT cells got segments in a little over one round.  us per step with those / these:
+    // 16 x (96 x 512) 48.3 / 32.7, 8 x (192 x 400) 30.7 / 21.5, 8 x 320^2 38.0 / 27.9
+    if (p->ty <= 0) p->ty = pick_segment_rows(g, rm.nown, tile_x, elem, sms, occ[launch_family(p)][0]);
     p->n_seg = (rm.nown + p->ty - 1) / p->ty;
     const long long items = (long long)p->n_strips * p->n_seg * g.n_cells;
     for (int fam = 0; fam < N_FAM; ++fam)
