@@ -120,11 +120,13 @@ def peaks():
 
 
 def source_digest():
-    """Digest of the fused kernel's code (comments and layout removed, so that
-    editing a comment does not orphan the committed DRAM counters)."""
+    """Digest of what decides the fused kernel's DRAM traffic: its code, and the
+    host side that chooses its form, segment height and L2 promotion (comments and
+    layout removed, so that editing a comment does not orphan the committed DRAM
+    counters)."""
     import re
     h = hashlib.sha256()
-    for f in ("lb_tiled.cuh", "lb_common.cuh", "lb_pair.cuh", "tma.cuh"):
+    for f in ("lb_tiled.cu", "lb_tiled.cuh", "lb_common.cuh", "lb_pair.cuh", "tma.cuh"):
         with open(os.path.join(ROOT, "paper_1004_5058_gb300", "csrc", f)) as fh:
             src = fh.read()
         src = re.sub(r"/\*.*?\*/", " ", src, flags=re.S)
