@@ -195,13 +195,13 @@ template <class C> __device__ inline C sin_pi(C x);
 template <> __device__ inline float sin_pi<float>(float x) { return sinpif(x); }
 template <> __device__ inline double sin_pi<double>(double x) { return sinpi(x); }
 
-// Body force density F_x of row y (zero when f0 = 0).
 // x == 0, FP64 by its bits: comparisons of doubles take the FP64 pipe's cycles too
 // (with the clamp of one_minus_exp_neg they were 6 of a thread's 265 operations per
 // row; without them 2048^2 takes 2.081 ms per step instead of 2.120)
 __device__ __forceinline__ bool is_zero(float x) { return x == 0.0f; }
 __device__ __forceinline__ bool is_zero(double x) { return (__double_as_longlong(x) << 1) == 0; }
 
+// Body force density F_x of row y (zero when f0 = 0).
 template <class C> __device__ inline C body_force_x(const ParamSet<C>& p, int y)
 {
     return is_zero(p.f0) ? C(0) : p.f0 * sin_pi<C>(C(y) * p.two_over_ny);
@@ -603,8 +603,10 @@ __device__ inline Sums<V> stencil_sums(const V d[12], const V e[4])
 // FP64, whose pipe bounds its kernels, folds the couplings into the stencil's
 // weights once per cell (ParamSet::gc, xc): ten operations fewer per site and
 // species.  With the table-driven psi, the reciprocals of lane_rcp and the tests of
-// density_ok a 2048^2 step took 2.50 ms before and takes 2.09; the errors against
-// 64-bit runs of the same starts are the same (ratios 0.93 .. 1.09 over 40 outputs).
+// density_ok a 2048^2 step took 2.50 ms before and takes 2.11.  Against 64-bit runs of
+// the same starts the fields' errors are the same on the whole (geometric mean of
+// their ratios 0.99 over 40 runs); single outputs of runs that amplify roundings lie
+// between 0.6 and 2.5 times theirs, both sides within 1e-12.
 template <class V> struct Pull {
     V gx, gy, xx, xy;
 };

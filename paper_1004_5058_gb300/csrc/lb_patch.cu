@@ -531,10 +531,13 @@ void patch_destroy(PatchPlan* p)
 // Patches of 32 x 8 sites (FP64: 16 x 8): 8 warps, so that a block hides some of
 // its own latency, and 0.7 (FP64: 0.9) halo sites per site.  Measured against 4,
 // 9, 12 and 16 rows and 8- and 16-column patches on 64^2 .. 512^2 cells: at 256^2
-// FP32 5.98 us per step against 9.4 (32 x 4) and 10.1 (16 x 8).  Below 10240 sites
-// FP64 takes 8 x 4 patches: 64^2 then has 128 of them, one for nearly every SM
-// (12.3 us against 19.6), whose FP64 pipes are the bound; above, 16 columns by the
-// 5 to 8 rows that spread best (256^2: 7 rows 44.8 us, 8 rows 49.6).
+// FP32 5.98 us per step against 9.4 (32 x 4) and 10.1 (16 x 8).  Up to 10240 sites
+// FP64 takes 8 x 4 patches: 64^2 then has 128 of them, one for nearly every SM, whose
+// FP64 pipes are the bound; above, 16 columns by the 5 to 8 rows that spread best
+// (256^2: 7 rows 44.8 us, 8 rows 49.6).  us per step, 8 x 4 / 16 columns: 32^2 9.6 /
+// 11.7, 64^2 11.2 / 12.1, 101 x 83 11.8 / 13.2, 96 x 106 12.7 / 13.2, 104^2 13.7 / 13.4,
+// 112^2 13.3 / 14.0, 120^2 14.9 / 13.8, 128^2 17.1 / 14.0; two cells of 64^2 13.2 / 12.3,
+// four 17.4 / 15.4.
 PatchPlan* patch_create(const Geom& g, int prec, int bc)
 {
     if (18 * g.plane >= (1LL << 31)) return nullptr;  // 32-bit element offsets inside a cell
