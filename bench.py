@@ -43,12 +43,12 @@ BYTES_PER_SITE = {"fp32": 144, "fp16": 72, "fp16sr": 72, "fp64": 288}
 FALLBACK_HBM_GBS = 6800.0
 # The FP64 step is bound by the FP64 pipe, not by HBM: its roofline counts the
 # FP64 pipe operations one site update issues (ncu counts of the fused tiled
-# kernel at tau = 1, the workload's: dfma 93, dadd 118, dmul 48 per site; each
+# kernel at tau = 1, the workload's: dfma 97, dadd 118, dmul 48 per site; each
 # occupies the pipe once) against the pipe's rate, 152 SMs x 2 FP64 operations
 # per clock (the nominal 1.25 TFLOP/s of FMA at the 2070 MHz maximum SM clock),
 # at the SM clock sampled in the run.  The count is the tiled kernel's; where
 # another kernel steps (step_form) the line reports no FP64 roofline.
-FP64_OPS_PER_SITE = 93 + 118 + 48
+FP64_OPS_PER_SITE = 97 + 118 + 48
 FP64_OPS_PER_CLOCK, N_SM, SM_MAX_MHZ = 2, 152, 2070.0
 
 

@@ -265,11 +265,11 @@ long long lb_steps_done(const lb_handle* h);
  * equals the run continued after lb_save bit for bit.  A file that is not a
  * checkpoint, is truncated or fails its checksum gives LB_ERR_INVALID and
  * leaves the handle without a loaded state.  Both calls are synchronous; the
- * file is binary in this machine's byte order (format version 2: a 128-byte
- * header, 15 float64 per cell, the float64 time sums, then the populations
+ * file is binary in this machine's byte order (format version 3: a 128-byte
+ * header, 19 float64 per cell, the float64 time sums, then the populations
  * [cell][s][i][y][x] without row padding, FNV-1a 64 checksum of the payload in
- * the header).  lb_load also reads version 1 files (14 float64 per cell, no
- * tau_b: one relaxation time). */
+ * the header).  lb_load also reads version 2 files (15 float64 per cell, no
+ * multiple-relaxation-time rates) and version 1 files (14, no tau_b either). */
 lb_status lb_save(lb_handle* h, const char* path);
 lb_status lb_load(lb_handle* h, const char* path);
 

@@ -23,8 +23,10 @@
 // Bound: latency.  A step is the chain flag -> populations -> densities -> collision
 // -> stores -> flag, two trips through L2 and a release that waits for the stores:
 // 3.2 us at 64^2 FP32 (a launch of the tiled kernel per step: 9.3 us with 8-row
-// segments, 6.0 with 2-row ones).  FP64 is bound by the FP64 pipe (64 cycles per
-// warp instruction on each sub-partition): 11 us at 64^2, 102 us before; two sites per thread took 19.3 us where one took 12.3.
+// segments, 6.0 with 2-row ones).  In FP64 that chain is long by its FP64 instructions,
+// 64 cycles each on a sub-partition: 11 us at 64^2 (102 before; the pipes 28 % busy,
+// two warps on an SM's four), 45 at 256^2, where the pipes fill; two sites per thread
+// took 19.3 us at 64^2 where one took 12.3.
 //
 // Steps are ordered by one flag per patch (the number of steps it has behind it):
 // a patch starts step s when all patches within three sites of it have finished
